@@ -357,7 +357,9 @@ fa_status fa_last_device_status(fa_ctx* ctx, fa_stream_t stream, int32_t* out);
 fa_status fa_set_wait_limits(fa_ctx* ctx, uint32_t loop_cap, uint64_t wait_ns);
 
 /* Raster schedule of this context's later frames (changes timing only, never
- * results).
+ * results).  By default a frame with sample-coverage marking is rasterized once (the
+ * depth pass keeps each pixel's triangle); conservative marking and FA_RASTER_HIZ
+ * rasterize a second time to mark, and mid_max_pix applies to them.
  *  mid_max_pix: a sub-triangle whose pixel box has at most 16 pixels is rasterized
  *    by one thread; larger ones are split into 16x16 tiles, one warp per tile.
  *    With mid_max_pix > 16, boxes of up to mid_max_pix pixels are also rasterized

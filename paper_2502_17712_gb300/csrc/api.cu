@@ -1,6 +1,7 @@
 // C ABI of libfastatlas: argument checks, context / mesh lifetime and the
 // stream-ordered launch sequences.  All compute happens in the kernels of the
 // other translation units.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -93,7 +94,7 @@ void fa_destroy(fa_ctx* ctx) {
   if (ctx->prof_on)
     for (int i = 0; i <= kMaxProf; ++i) cudaEventDestroy(ctx->prof_ev[i]);
   const PackScratch& p = ctx->pack;
-  void* ptrs[] = {ctx->ctr, ctx->zbuf, ctx->zmax, ctx->queue, ctx->tile_owner, ctx->cand, ctx->surv, ctx->surv_count, ctx->surv_clip, ctx->clip, ctx->clip_count,
+  void* ptrs[] = {ctx->ctr, ctx->zbuf, ctx->ties, ctx->zmax, ctx->queue, ctx->tile_owner, ctx->cand, ctx->surv, ctx->surv_count, ctx->surv_clip, ctx->clip, ctx->clip_count,
                   ctx->label, ctx->wordroots, ctx->blockcnt, ctx->viscnt, ctx->vis, ctx->xedge, ctx->xcnt, ctx->tile_flag, ctx->tile_list,
                   ctx->box_enc, ctx->box_full, p.ord_counts, p.ord_rank, p.ord_total,
                   p.order, p.fs, p.rec8, p.segs, p.scan_state, p.m, p.xy, p.cand, ctx->psched};
@@ -140,7 +141,9 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
 #define FA_ALLOC(ptr, n) \
   if (st == FA_OK) st = alloc(&ptr, (size_t)(n));
   FA_ALLOC(ctx->ctr, 1);
-  FA_ALLOC(ctx->zbuf, (uint64_t)c.max_width * c.max_height);
+  FA_ALLOC(ctx->zbuf, 2ull * c.max_width * c.max_height);
+  ctx->tie_cap = (uint32_t)std::max<uint64_t>(4096u, (uint64_t)c.max_width * c.max_height);
+  FA_ALLOC(ctx->ties, ctx->tie_cap);
   FA_ALLOC(ctx->zmax, (uint64_t)((c.max_width + 15) / 16) * ((c.max_height + 15) / 16));
   FA_ALLOC(ctx->queue, ctx->queue_cap);
   ctx->tile_cap = 4u * ctx->queue_cap;

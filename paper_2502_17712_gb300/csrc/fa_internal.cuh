@@ -35,6 +35,8 @@ constexpr uint32_t kMaxFrontBlocks = 152 * 4;  // raster front-end blocks (survi
 constexpr uint32_t kDefaultPushThreads = 512;  // threads of a candidate's push CTA (fa_set_chart_pack_schedule)
 constexpr uint32_t kPschedWords = 64;          // schedule state of a single-view persistent launch
 
+constexpr int kMidLists = 32;  // lists of mid-size sub-triangles (one counter each, so that few warps share one)
+
 struct DevCounters {
   int32_t status;          // sticky fa_status of the context
   uint32_t pad0;
@@ -47,6 +49,8 @@ struct DevCounters {
   uint32_t n_vis;          // entries of the visible-triangle list
   uint32_t n_vtiles;       // 1024-triangle tiles with a visible triangle (listed by the marking pass)
   uint32_t uf_item;        // next listed tile of the local union-find
+  uint32_t n_ties;         // equal depth keys listed by the depth pass
+  uint32_t n_mid[kMidLists][32];  // [.][0]: mid-size sub-triangles of each list (a line each)
 };
 
 // One queued (large) sub-triangle of the raster: snapped vertices, depths and its
@@ -113,7 +117,9 @@ struct fa_ctx {
   const char* prof_name[kMaxProf];
   // scratch
   fa::DevCounters* ctr;
-  uint32_t* zbuf;        // [max_w * max_h]
+  uint32_t* zbuf;        // [max_w * max_h] depth keys, or 64-bit key | triangle
+  uint4* ties;           // [tie_cap] pixels where two triangles have the same key
+  uint32_t tie_cap;
   uint32_t* zmax;        // [ceil(max_w / 16) * ceil(max_h / 16)] largest depth key per 16x16 tile
   uint32_t* tile_flag;   // [ceil(max_tris / 1024)] tile has a visible triangle (this frame)
   uint32_t* tile_list;   // [ceil(max_tris / 1024)] those tiles, in the order the marking found them

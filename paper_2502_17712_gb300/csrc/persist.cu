@@ -126,11 +126,19 @@ template <bool DEV_M>
 __device__ __noinline__ void st_exact(const ViewArgs& v, uint32_t j, uint32_t n) {
   rs::exact_body<DEV_M, kPT>(v.ra, j, n);
 }
+template <bool DEV_M>
+__device__ __noinline__ void st_exact_win(const ViewArgs& v, uint32_t j, uint32_t n) {
+  rs::exact_win_body<DEV_M, kPT>(v.ra, j, n);
+}
 __device__ __noinline__ void st_depth_big(const ViewArgs& v, uint32_t j, uint32_t n) { rs::depth_big_body(v.ra, j, n); }
+__device__ __noinline__ void st_depth_win(const ViewArgs& v, uint32_t j, uint32_t n) { rs::depth_win_body(v.ra, j, n); }
 __device__ __noinline__ void st_zmax(const ViewArgs& v, uint32_t j, uint32_t n) { rs::zmax_body(v.ra, j, n); }
 template <bool CONS>
 __device__ __noinline__ void st_mark(const ViewArgs& v, uint32_t j, uint32_t n) {
   rs::mark_body<CONS, kPT>(v.ra, j, n);
+}
+__device__ __noinline__ void st_mark_win(const ViewArgs& v, uint32_t j, uint32_t n) {
+  rs::mark_win_body<kPT>(v.ra, j, n);
 }
 __device__ __noinline__ void st_init_v(const ViewArgs& v, uint32_t j, uint32_t n) {
   cf::init_v_body(v.uf.label, v.uf.T, v.uf.V, j, n);
@@ -192,18 +200,21 @@ __device__ __forceinline__ void run_stage_inline(const ViewArgs& v, uint32_t sta
   // (the device-matrix and conservative variants, and the other stages, keep their
   // own register allocation in the non-inlined wrappers)
   if (stage == S_FRONT && !v.devm) rs::front_body<false>(v.ra, j, n);
-  else if (stage == S_EXACT && !v.devm) rs::exact_body<false, kPT>(v.ra, j, n);
-  else if (stage == S_MARK && !v.cons) rs::mark_body<false, kPT>(v.ra, j, n);
+  else if (stage == S_EXACT && !v.devm && v.ra.win) rs::exact_win_body<false, kPT>(v.ra, j, n);
+  else if (stage == S_DEPTH_BIG && v.ra.win) rs::depth_win_body(v.ra, j, n);
   else run_stage(v, stage, j, n, smem);
 }
 
 __device__ void run_stage(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_t n, unsigned char* smem) {
   switch (stage) {
     case S_FRONT: v.devm ? st_front<true>(v, j, n) : st_front<false>(v, j, n); break;
-    case S_EXACT: v.devm ? st_exact<true>(v, j, n) : st_exact<false>(v, j, n); break;
-    case S_DEPTH_BIG: st_depth_big(v, j, n); break;
+    case S_EXACT:
+      if (v.ra.win) v.devm ? st_exact_win<true>(v, j, n) : st_exact_win<false>(v, j, n);
+      else v.devm ? st_exact<true>(v, j, n) : st_exact<false>(v, j, n);
+      break;
+    case S_DEPTH_BIG: v.ra.win ? st_depth_win(v, j, n) : st_depth_big(v, j, n); break;
     case S_ZMAX: st_zmax(v, j, n); break;
-    case S_MARK: v.cons ? st_mark<true>(v, j, n) : st_mark<false>(v, j, n); break;
+    case S_MARK: v.ra.win ? st_mark_win(v, j, n) : v.cons ? st_mark<true>(v, j, n) : st_mark<false>(v, j, n); break;
     case S_INIT_V: st_init_v(v, j, n); break;
     case S_LOCAL: st_local(v, j, n); break;
     case S_HOOK: st_hook(v, j, n); break;
@@ -385,6 +396,7 @@ void build_view(fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params* p, cons
   // (twice the front end's workers: a small frame's survivors then get the raster's
   // lane groups, one group per survivor)
   const uint32_t n_rast = wk(T, 64);
+  rs::set_exact_grid(v.ra, n_rast, kPT);
   add(S_EXACT, n_rast);
   add(S_DEPTH_BIG, n_pix);
   if (v.ra.zmax) add(S_ZMAX, wk(pix, 8192));
@@ -583,6 +595,7 @@ fa_status plan_build(fa_batch_plan* pl) {
         vps[i].workers[q] = (uint32_t)std::min<uint64_t>(pl->G, std::max<uint64_t>(1, (pix + 8191) / 8192));
         ++vps[i].n_stages;
       }
+      fa::rs::set_raster_mode(vps[i].va.ra);
       va[i] = vps[i].va;
       front_cap = std::max(front_cap, vps[i].front_cap);
     }

@@ -16,15 +16,18 @@ __global__ void __launch_bounds__(rs::kFrontThreads, 2) k_raster_front(RasterArg
   rs::front_body<DEV_M>(A, blockIdx.x, gridDim.x);
 }
 
-template <bool DEV_M>
+template <bool DEV_M, bool WIN>
 __global__ void __launch_bounds__(256, 4) k_raster_exact(RasterArgs A) {
   pdl_wait();
-  rs::exact_body<DEV_M, 256>(A, blockIdx.x, gridDim.x);
+  if (WIN) rs::exact_win_body<DEV_M, 256>(A, blockIdx.x, gridDim.x);
+  else rs::exact_body<DEV_M, 256>(A, blockIdx.x, gridDim.x);
 }
 
+template <bool WIN>
 __global__ void __launch_bounds__(256) k_raster_depth_big(RasterArgs A) {
   pdl_wait();
-  rs::depth_big_body(A, blockIdx.x, gridDim.x);
+  if (WIN) rs::depth_win_body(A, blockIdx.x, gridDim.x);
+  else rs::depth_big_body(A, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(256) k_raster_zmax(RasterArgs A) {
@@ -32,10 +35,13 @@ __global__ void __launch_bounds__(256) k_raster_zmax(RasterArgs A) {
   rs::zmax_body(A, blockIdx.x, gridDim.x);
 }
 
-template <bool CONS>
+enum MarkMode { kMarkSamples, kMarkConservative, kMarkWinners };
+
+template <int MODE>
 __global__ void __launch_bounds__(256, 4) k_raster_mark(RasterArgs A) {
   pdl_wait();
-  rs::mark_body<CONS, 256>(A, blockIdx.x, gridDim.x);
+  if (MODE == kMarkWinners) rs::mark_win_body<256>(A, blockIdx.x, gridDim.x);
+  else rs::mark_body<MODE == kMarkConservative, 256>(A, blockIdx.x, gridDim.x);
 }
 
 }  // namespace
@@ -48,32 +54,33 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
   // (and enough blocks for the clears: at most 16 depth-buffer pixels per thread)
   const uint32_t fb = std::max(grid_for(mesh->T, rs::kFrontThreads, 152u * 2u),
                                grid_for((uint64_t)W * H, rs::kFrontThreads * 16u, 152u * 2u));
-  const RasterArgs A = rs::make_raster_args(ctx, mesh, M, W, H, vt, reset_status, Mdev, cons, tri_chart_init, fb,
-                                            rs::kFrontThreads);
-  ctx->front_blocks = A.front_blocks;
   const unsigned gb = 152 * 8;
+  RasterArgs A = rs::make_raster_args(ctx, mesh, M, W, H, vt, reset_status, Mdev, cons, tri_chart_init, fb,
+                                            rs::kFrontThreads);
+  rs::set_exact_grid(A, gb, 256);
+  ctx->front_blocks = A.front_blocks;
   mark(ctx, "k_raster_front", s);
   if (Mdev)
     launch_k(k_raster_front<true>, A.front_blocks, rs::kFrontThreads, 0, s, A);
   else
     launch_k(k_raster_front<false>, A.front_blocks, rs::kFrontThreads, 0, s, A);
   mark(ctx, "k_raster_exact", s);
-  if (Mdev)
-    launch_k(k_raster_exact<true>, 152 * 8, 256, 0, s, A);
+  if (A.win)
+    launch_k(Mdev ? k_raster_exact<true, true> : k_raster_exact<false, true>, gb, 256, 0, s, A);
   else
-    launch_k(k_raster_exact<false>, 152 * 8, 256, 0, s, A);
+    launch_k(Mdev ? k_raster_exact<true, false> : k_raster_exact<false, false>, gb, 256, 0, s, A);
   mark(ctx, "k_raster_depth_big", s);
-  launch_k(k_raster_depth_big, gb, 256, 0, s, A);
+  launch_k(A.win ? k_raster_depth_big<true> : k_raster_depth_big<false>, gb, 256, 0, s, A);
   if (A.zmax) {
     mark(ctx, "k_raster_zmax", s);
     launch_k(k_raster_zmax, grid_for((uint64_t)A.ztx * ((H + 15) / 16) * 32, 256, 152 * 8), 256, 0, s, A);
   }
   mark(ctx, "k_raster_mark", s);
   // one wave of four resident blocks per SM: each block scans the region counts once
-  if (cons)
-    launch_k(k_raster_mark<true>, 152 * 4, 256, 0, s, A);
+  if (A.win)  // (blocks of 64 x 32 pixels)
+    launch_k(k_raster_mark<kMarkWinners>, std::min(((W + 63) / 64) * ((H + 31) / 32), 152u * 8u), 256, 0, s, A);
   else
-    launch_k(k_raster_mark<false>, 152 * 4, 256, 0, s, A);
+    launch_k(cons ? k_raster_mark<kMarkConservative> : k_raster_mark<kMarkSamples>, 152 * 4, 256, 0, s, A);
   FA_CUDA_TRY(cudaGetLastError());
   return FA_OK;
 }

@@ -15,11 +15,14 @@
 // Kernels: k_raster_front (the per-triangle front end above; it also clears the
 // per-frame state for the kernels after it), k_raster_exact (the exact set-up of
 // the survivors; small sub-triangles rasterized in-thread, or by a group of 16
-// lanes each when the survivors are few for the grid, a 48-byte record kept for the
-// marking pass), k_raster_depth_big (the queued tiles) and k_raster_mark (the queued
-// tiles, then the records, grouped in the same way; it also lists the 1024-triangle
-// tiles that hold a visible triangle for the chart passes).  Edge values that stay
-// below 2^24 over a box are stepped as exact fp32 integers.
+// lanes each when the survivors are few for the grid), k_raster_depth_big (the larger
+// ones) and k_raster_mark (the visible bits; it also lists the 1024-triangle tiles
+// that hold a visible triangle for the chart passes).  Two forms of the last three:
+// "winners" (the default; below), where the depth pass keeps each pixel's triangle, and
+// two rasterizations (conservative marking, the tile-depth option), where the exact
+// pass keeps a 48-byte record of each small sub-triangle and the marking pass
+// rasterizes the queued tiles and the records again.  Edge values that stay below 2^24
+// over a box are there stepped as exact fp32 integers.
 #pragma once
 #include "fa_internal.cuh"
 
@@ -332,6 +335,12 @@ struct RasterArgs {
   uint32_t* clip;  // triangles that need clipping, one region per front block like surv
   DevCounters* ctr;
   uint32_t* vt;
+  // single-pass visibility (see "winners" below): the depth buffer holds key << 32 | triangle
+  int win;
+  unsigned long long* zid;  // [W * H], the same memory as zbuf
+  uint4* ties;              // [tie_cap] (pixel, key, triangle, triangle) of equal keys
+  uint32_t tie_cap;
+  uint32_t mid_blocks, mid_lists, mid_per_block;  // exact pass's blocks, mid-size lists, slots per block
 };
 
 __device__ __forceinline__ CandTri make_cand(const SV& a, const SV& b, const SV& c, const Setup& s, uint32_t t) {
@@ -560,11 +569,14 @@ __device__ __forceinline__ void front_body(const RasterArgs& A, uint32_t bid, ui
       A.ctr->ncand = 0u;
       A.ctr->n_vtiles = 0u;
       A.ctr->uf_item = 0u;
+      A.ctr->n_ties = 0u;
     }
   }
+  if (bid == 0 && threadIdx.x < kMidLists) A.ctr->n_mid[threadIdx.x][0] = 0u;
   {
     const uint32_t gstride = nblk * blockDim.x, g0 = bid * blockDim.x + threadIdx.x;
-    const uint32_t npix = (uint32_t)A.W * (uint32_t)A.H, n4 = npix / 4, nwords = (A.T + 31) / 32;
+    const uint32_t npix = ((uint32_t)A.W * (uint32_t)A.H) << (A.win ? 1 : 0);  // 32-bit words of the depth buffer
+    const uint32_t n4 = npix / 4, nwords = (A.T + 31) / 32;
     uint4* z4 = reinterpret_cast<uint4*>(A.zbuf);
     const uint4 ff = make_uint4(0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu);
     for (uint32_t i = g0; i < n4; i += gstride) z4[i] = ff;
@@ -628,6 +640,12 @@ __device__ __forceinline__ void front_body(const RasterArgs& A, uint32_t bid, ui
     A.surv_count[bid] = s_count;
     A.clip_count[bid] = s_nclip;
   }
+}
+
+// The shared words of region_prefix, one array for all bodies of a kernel.
+__device__ __forceinline__ uint32_t* region_pre() {
+  __shared__ uint32_t pre[kMaxFrontBlocks + 1];
+  return pre;
 }
 
 // Exclusive prefix of the front blocks' per-region counts (survivors or clipped
@@ -745,7 +763,7 @@ __device__ __forceinline__ bool group_raster(const SV& a0, const SV& b0, const S
 // triangles append theirs after slot T.
 template <bool DEV_M, int NT>
 __device__ __forceinline__ void exact_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
-  __shared__ uint32_t pre[kMaxFrontBlocks + 1];
+  uint32_t* pre = region_pre();
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t n = surv_prefix<NT>(A, pre);
   const uint32_t stride = nblk * blockDim.x;
@@ -982,7 +1000,7 @@ __device__ __forceinline__ void big_tiles(const RasterArgs& A, uint32_t bid, uin
 // that finish their share of the tiles early take candidate records.
 template <bool CONS, int NT>
 __device__ __forceinline__ void mark_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
-  __shared__ uint32_t pre[kMaxFrontBlocks + 1];
+  uint32_t* pre = region_pre();
   __shared__ int32_t s_status;
   if (threadIdx.x == 0) s_status = __ldcg(&A.ctr->status);
   __syncthreads();
@@ -1055,6 +1073,659 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
   big_tiles<0>(A, bid, nblk);
 }
 
+// ------------------------------------------------------------------ winners
+//
+// Single-pass visibility (sample-coverage marking; the default).  A sample of the
+// marking pass passes "<=" exactly when its key equals the pixel's smallest key, and
+// both passes take the same samples, so the triangles to mark are those that own a
+// pixel's smallest key: the depth pass keeps key << 32 | triangle per pixel (64-bit
+// atomicMin) and the marking pass is one read of that buffer instead of a second
+// rasterization.  Two triangles with the same key at a pixel are told by the returned
+// old value: the key a pixel ends with stays there once it has arrived, so every later
+// triangle with that key sees it and lists the pair; the marking pass marks the pairs
+// whose key is still the pixel's.  If the list overflows, the marking pass tests every
+// survivor against the buffer instead (mark_all).
+//
+// Three sizes of sub-triangles, so that the lanes of a warp have like work: boxes of at
+// most kSmallMaxPix pixels are rasterized where they are set up (exact pass); boxes of
+// at most kMidPix are listed and then rasterized by 1 .. 16 lanes each, as many as fill
+// the grid, a lane taking whole rows; larger ones are 16x16 tiles, a warp per tile.
+// Edge functions of sub-triangles of less than 96 pixels a side fit 32 bits (twice
+// the product of the sides is below 2^31, also 16 pixels past the box); their conversions to fp32 round as the 64-bit
+// ones do.  A top-left edge passes at 0, another one from 1, so that with 1 taken from
+// the others a sample is covered when no value is negative.
+//
+// What bounds it: the atomics' round trips and, on views of many mid-size triangles,
+// their issue (about 120 G samples/s).  Four samples of a lane are on their way at once
+// (one: 851 us for the larger boxes of a 3.2M-triangle floor at 1440p; four: 379;
+// eight spill: 999) and at least four lanes share a box, so that their atomics meet in
+// a sector (one lane: 446 us, two 384, four 374, eight 420).  A load of the pixel's key
+// before the atomic costs more than the atomics it saves (471 us).  Against two
+// rasterizations, exact + larger boxes + marking: that floor 2475 -> 551 us, a floor of
+// 60 patches at 1080p 247 -> 89, 200 icospheres at 1080p 107 -> 63, one patch of
+// 7,938 triangles at 1080p 52 -> 43 (events around each kernel, GB300).
+constexpr int kMidPix = 256;  // (512: the same)
+constexpr uint32_t kMinLanes = 2;  // log2 of the fewest lanes a mid-size box gets
+constexpr int kSpan32 = 96 * kSub;  // side of a sub-triangle with 32-bit edge functions
+
+struct Tri32 {
+  int X[3], Y[3];
+  float z[3];
+};
+
+// Snapped vertices, pixel box and size class of one unclipped triangle.
+struct WinSetup {
+  Tri32 v;
+  int px0, py0, px1, py1;
+  bool fits;  // 32-bit edge functions
+  bool live;  // front facing, with a sample in its box
+};
+
+__device__ __forceinline__ void project32(const float4& c, float hx, float hy, int& X, int& Y, float& z) {
+  const SV s = project(CV{c.x, c.y, c.z, c.w}, hx, hy);
+  X = (int)s.X;
+  Y = (int)s.Y;
+  z = s.zn;
+}
+
+__device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4& c0, const float4& c1,
+                                              const float4& c2) {
+  WinSetup s;
+  project32(c0, A.hx, A.hy, s.v.X[0], s.v.Y[0], s.v.z[0]);
+  project32(c1, A.hx, A.hy, s.v.X[1], s.v.Y[1], s.v.z[1]);
+  project32(c2, A.hx, A.hy, s.v.X[2], s.v.Y[2], s.v.z[2]);
+  const int xmn = min(s.v.X[0], min(s.v.X[1], s.v.X[2])), xmx = max(s.v.X[0], max(s.v.X[1], s.v.X[2]));
+  const int ymn = min(s.v.Y[0], min(s.v.Y[1], s.v.Y[2])), ymx = max(s.v.Y[0], max(s.v.Y[1], s.v.Y[2]));
+  s.px0 = max(-((128 - xmn) >> 8), 0);
+  s.px1 = min((xmx - 128) >> 8, A.W - 1);
+  s.py0 = max(-((128 - ymn) >> 8), 0);
+  s.py1 = min((ymx - 128) >> 8, A.H - 1);
+  s.fits = xmx - xmn < kSpan32 && ymx - ymn < kSpan32;
+  const int ux = s.v.X[1] - s.v.X[0], uy = s.v.Y[1] - s.v.Y[0], vx = s.v.X[2] - s.v.X[0], vy = s.v.Y[2] - s.v.Y[0];
+  const bool front = s.fits ? ux * vy - vx * uy > 0 : (int64_t)ux * vy - (int64_t)vx * uy > 0;
+  s.live = front && s.px1 >= s.px0 && s.py1 >= s.py0;
+  return s;
+}
+
+__device__ __forceinline__ void note_tie(const RasterArgs& A, uint32_t pix, uint32_t key, uint32_t t0, uint32_t t1) {
+  const uint32_t i = atomicAdd(&A.ctr->n_ties, 1u);
+  if (i < A.tie_cap) A.ties[i] = make_uint4(pix, key, t0, t1);
+}
+
+// The samples a thread has put: the returned value of one is looked at when the next
+// is on its way.
+struct Put {
+  unsigned long long old = ~0ull;
+  uint32_t key = 0u, pix = 0u;
+  __device__ __forceinline__ void check(const RasterArgs& A, uint32_t t) const {
+    if ((uint32_t)(old >> 32) == key && (uint32_t)old != t) note_tie(A, pix, key, (uint32_t)old, t);
+  }
+  __device__ __forceinline__ void put(const RasterArgs& A, uint32_t p, uint32_t k, uint32_t t) {
+    const unsigned long long o = atomicMin(A.zid + p, ((unsigned long long)k << 32) | t);
+    check(A, t);
+    old = o;
+    key = k;
+    pix = p;
+  }
+};
+
+// Edge functions at the sample of pixel (px, py), their steps per pixel, and the plane's
+// weights of a 32-bit sub-triangle.
+struct Edges32 {
+  int e[3], dx[3], dy[3], nb[3];  // e: less nb (0: top-left edge, 1: another)
+  float invA;
+};
+
+__device__ __forceinline__ Edges32 edges32(const Tri32& v, int px, int py) {
+  Edges32 E;
+  const int sx = px * 256 + 128, sy = py * 256 + 128;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int a = (i + 1) % 3, b = (i + 2) % 3;  // E0: edge v1 -> v2, E1: v2 -> v0, E2: v0 -> v1
+    const int ex = v.X[b] - v.X[a], ey = v.Y[b] - v.Y[a];
+    E.nb[i] = (ey < 0 || (ey == 0 && ex < 0)) ? 0 : 1;
+    E.e[i] = ex * (sy - v.Y[a]) - ey * (sx - v.X[a]) - E.nb[i];
+    E.dx[i] = -ey * 256;
+    E.dy[i] = ex * 256;
+  }
+  const int area = (v.X[1] - v.X[0]) * (v.Y[2] - v.Y[0]) - (v.X[2] - v.X[0]) * (v.Y[1] - v.Y[0]);
+  E.invA = __fdiv_rn(1.0f, __int2float_rn(area));
+  return E;
+}
+
+// Depth key of a covered sample with (reduced) edge values e; false outside [-1, 1].
+__device__ __forceinline__ bool key32(const Edges32& E, int e0, int e1, int e2, const Tri32& v, uint32_t& key) {
+  float s = __fmul_rn(__int2float_rn(e0 + E.nb[0]), v.z[0]);
+  s = __fadd_rn(s, __fmul_rn(__int2float_rn(e1 + E.nb[1]), v.z[1]));
+  s = __fadd_rn(s, __fmul_rn(__int2float_rn(e2 + E.nb[2]), v.z[2]));
+  const float d = __fmul_rn(s, E.invA);
+  key = ordered(d);
+  return d >= -1.0f && d <= 1.0f;
+}
+
+__device__ __forceinline__ uint32_t zkey(const RasterArgs& A, uint32_t pix) {
+  return __ldcg(reinterpret_cast<const uint32_t*>(A.zid) + 2 * (size_t)pix + 1);
+}
+
+// A thread's N samples on their way: keys put, and the old values of the N before them,
+// which are looked at once these are issued.
+template <int N>
+struct PutN {
+  unsigned long long old[N];
+  uint32_t key[N], pix[N];
+  __device__ __forceinline__ PutN() {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      old[i] = ~0ull;
+      key[i] = pix[i] = 0u;
+    }
+  }
+  __device__ __forceinline__ void check(const RasterArgs& A, uint32_t t) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if ((uint32_t)(old[i] >> 32) == key[i] && (uint32_t)old[i] != t) note_tie(A, pix[i], key[i], (uint32_t)old[i], t);
+  }
+  __device__ __forceinline__ void put(const RasterArgs& A, uint32_t t, const bool (&on)[N], const uint32_t (&k)[N],
+                                      const uint32_t (&p)[N]) {
+    unsigned long long o[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      o[i] = on[i] ? atomicMin(A.zid + p[i], ((unsigned long long)k[i] << 32) | t) : ~0ull;
+    check(A, t);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      old[i] = o[i];
+      key[i] = on[i] ? k[i] : 0u;
+      pix[i] = p[i];
+    }
+  }
+};
+
+// Samples first, first + step, .. (row order) of a 32-bit sub-triangle's box, N at a time
+// so that their atomics overlap.  step lanes side by side then put neighbouring pixels.
+template <int N>
+__device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uint32_t t, int px0, int py0, int px1,
+                                        int py1, int first, int step) {
+  const int w = px1 - px0 + 1, n = w * (py1 - py0 + 1);
+  if (first >= n) return;
+  const int sy = step == 1 ? (w == 1 ? 1 : 0) : step / w, sx = step - sy * w;  // step = sy rows and sx < w pixels
+  const int fy = first / w, fx = first - fy * w;
+  const Edges32 E = edges32(v, px0 + fx, py0 + fy);
+  // a step inside the row, and one that runs past its end (a row more, w pixels back)
+  const int a0 = E.dy[0] * sy + E.dx[0] * sx, a1 = E.dy[1] * sy + E.dx[1] * sx, a2 = E.dy[2] * sy + E.dx[2] * sx;
+  const int b0 = a0 + E.dy[0] - E.dx[0] * w, b1 = a1 + E.dy[1] - E.dx[1] * w, b2 = a2 + E.dy[2] - E.dx[2] * w;
+  const uint32_t ap = (uint32_t)(A.W * sy + sx), bp = ap + (uint32_t)(A.W - w);
+  int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2], col = w - fx;  // col: pixels to the row's end
+  uint32_t p = (uint32_t)(py0 + fy) * (uint32_t)A.W + (uint32_t)(px0 + fx);
+  PutN<N> q;
+  for (int s = first; s < n;) {
+    uint32_t key[N], pix[N];
+    bool on[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      pix[i] = p;
+      on[i] = (e0 | e1 | e2) >= 0 && s < n && key32(E, e0, e1, e2, v, key[i]);
+      col -= sx;
+      const bool wrap = col <= 0;
+      col += wrap ? w : 0;
+      e0 += wrap ? b0 : a0;
+      e1 += wrap ? b1 : a1;
+      e2 += wrap ? b2 : a2;
+      p += wrap ? bp : ap;
+      s += step;
+    }
+    q.put(A, t, on, key, pix);
+  }
+  q.check(A, t);
+}
+
+// Any sub-triangle, 64-bit edge functions: samples first, first + step, .. of its box in
+// row order.  TEST: nothing is written; true when one of them has the pixel's final key.
+template <bool TEST>
+__device__ __forceinline__ bool win_rect64(const RasterArgs& A, const SV& a, const SV& b, const SV& c, uint32_t t, int px0,
+                                           int py0, int px1, int py1, uint32_t first, uint32_t step) {
+  const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
+  const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
+  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
+  Put q;
+  for (uint32_t s = first; s < n; s += step) {
+    const int px = px0 + (int)(s % w), py = py0 + (int)(s / w);
+    const Edges E = edges_at(a, b, c, px, py);
+    const bool in = (E.e[0] > 0 || (E.e[0] == 0 && E.tl[0])) && (E.e[1] > 0 || (E.e[1] == 0 && E.tl[1])) &&
+                    (E.e[2] > 0 || (E.e[2] == 0 && E.tl[2]));
+    if (!in) continue;
+    float f = __fmul_rn(ll2float_rn(E.e[0]), a.zn);
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[1]), b.zn));
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[2]), c.zn));
+    const float d = __fmul_rn(f, invA);
+    if (!(d >= -1.0f && d <= 1.0f)) continue;
+    const uint32_t key = ordered(d), p = (uint32_t)py * (uint32_t)A.W + (uint32_t)px;
+    if (TEST) {
+      if (key <= zkey(A, p)) return true;
+    } else {
+      q.put(A, p, key, t);
+    }
+  }
+  if (!TEST) q.check(A, t);
+  return false;
+}
+
+// One queue record and its tiles for a large sub-triangle, at (entry e, first tile):
+// false when the queue or the tile table is full (the reserved record is then empty and
+// the reserved tiles have no owner).
+__device__ __forceinline__ bool win_queue(const RasterArgs& A, const int (&X)[3], const int (&Y)[3],
+                                          const float (&z)[3], int px0, int py0, int px1, int py1, bool fits,
+                                          uint32_t t, uint64_t e, uint64_t tile, uint32_t tiles) {
+  const bool ok = e < A.queue_cap && tile + tiles <= A.tile_cap;
+  if (e < A.queue_cap) {
+    BigTri bt;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      bt.X[i] = X[i];
+      bt.Y[i] = Y[i];
+      bt.zn[i] = z[i];
+    }
+    bt.px0 = ok ? px0 : 1;
+    bt.py0 = ok ? py0 : 1;
+    bt.px1 = ok ? px1 : 0;
+    bt.py1 = ok ? py1 : 0;
+    bt.tri = t;
+    bt.tile0 = (uint32_t)tile;
+    bt.pad = fits ? 1u : 0u;
+    A.queue[e] = bt;
+  }
+  for (uint64_t j = tile; j < tile + tiles && j < A.tile_cap; ++j) A.tile_owner[j] = ok ? (uint32_t)e : 0xFFFFFFFFu;
+  return ok;
+}
+
+__device__ __forceinline__ uint32_t tiles_of(int w, int h) {
+  return (uint32_t)((w + kBigTile - 1) / kBigTile) * (uint32_t)((h + kBigTile - 1) / kBigTile);
+}
+
+// A triangle that must be clipped (rare).  TEST as in win_rect64; else its sub-triangles
+// are rasterized here (small) or queued.
+template <bool TEST>
+__device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4 c0, float4 c1, float4 c2) {
+  CV poly[kMaxPoly];
+  poly[0] = CV{c0.x, c0.y, c0.z, c0.w};
+  poly[1] = CV{c1.x, c1.y, c1.z, c1.w};
+  poly[2] = CV{c2.x, c2.y, c2.z, c2.w};
+  const int n = clip_polygon(poly, 3);
+  if (n < 0) {
+    if (!TEST) set_status(A.ctr, FA_E_CAPACITY);
+    return false;
+  }
+  if (n < 3) return false;
+  for (int i = 0; i < n; ++i)
+    if (!(poly[i].w > 0.0f)) return false;
+  SV sv[kMaxPoly];
+  for (int i = 0; i < n; ++i) sv[i] = project(poly[i], A.hx, A.hy);
+  for (int i = 1; i + 1 < n; ++i) {
+    const SV &a = sv[0], &b = sv[i], &c = sv[i + 1];
+    const Setup s = setup(a, b, c, A.W, A.H, false);
+    if (s.A <= 0 || s.px1 < s.px0 || s.py1 < s.py0) continue;
+    if (TEST) {
+      if (win_rect64<true>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u)) return true;
+      continue;
+    }
+    const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
+    if (w * h > kSmallMaxPix) {
+      const uint32_t tiles = tiles_of(w, h);
+      const unsigned long long old = atomicAdd(&A.ctr->big, (1ull << 40) | (unsigned long long)tiles);
+      const int X[3] = {(int)a.X, (int)b.X, (int)c.X}, Y[3] = {(int)a.Y, (int)b.Y, (int)c.Y};
+      const float z[3] = {a.zn, b.zn, c.zn};
+      if (win_queue(A, X, Y, z, s.px0, s.py0, s.px1, s.py1, false, t, old >> 40, old & ((1ull << 40) - 1), tiles))
+        continue;
+    }
+    win_rect64<false>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u);
+  }
+  return false;
+}
+
+// First slot of mid-size list r (its blocks' shares one after the other).
+__device__ __forceinline__ uint32_t mid_base(const RasterArgs& A, uint32_t r) {
+  return (uint32_t)((uint64_t)r * A.mid_blocks / A.mid_lists) * A.mid_per_block;
+}
+
+// Exact set-up of the survivors (as exact_body): small ones rasterized here, mid-size
+// ones listed, large ones queued.
+template <bool DEV_M, int NT>
+__device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  uint32_t* pre = region_pre();
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t n = surv_prefix<NT>(A, pre);
+  const uint32_t stride = nblk * blockDim.x;
+  const bool grouped = (uint64_t)n * kRasterGroup <= (uint64_t)stride;  // few survivors: see exact_body
+  const uint32_t sub = lane & (kRasterGroup - 1u);
+  const uint32_t list = ((bid + 1u) * A.mid_lists - 1u) / A.mid_blocks;
+  const uint32_t lbase = mid_base(A, list), lcap = mid_base(A, list + 1u) - lbase;
+  for (uint32_t wbase = bid * blockDim.x + (threadIdx.x & ~31u); (grouped ? wbase / kRasterGroup : wbase) < n;
+       wbase += stride) {
+    const uint32_t vfirst = grouped ? wbase / kRasterGroup : wbase;
+    const uint32_t v = grouped ? (sub == 0u ? vfirst + lane / kRasterGroup : n) : wbase + lane;
+    WinSetup E = {};
+    uint32_t t = 0, tiles = 0;
+    int kind = 0;  // 0 nothing, 1 small, 2 large, 3 mid-size
+    if (v < n) {
+      const uint32_t i = surv_slot(A, pre, v, vfirst);
+      const float4* sc = A.surv_clip + 3 * (size_t)i;
+      t = __ldcg(A.surv + i);
+      E = win_setup(A, __ldcs(sc), __ldcs(sc + 1), __ldcs(sc + 2));
+      if (E.live) {
+        const int w = E.px1 - E.px0 + 1, h = E.py1 - E.py0 + 1, pix = w * h;
+        kind = !E.fits ? 2 : pix <= kSmallMaxPix ? 1 : pix <= kMidPix ? 3 : 2;
+        if (kind == 2) tiles = tiles_of(w, h);
+      }
+    }
+    const uint32_t mids = __ballot_sync(0xFFFFFFFFu, kind == 3);
+    if (mids) {
+      uint32_t o = 0;
+      if (lane == 0) o = atomicAdd(&A.ctr->n_mid[list][0], (uint32_t)__popc(mids));
+      o = __shfl_sync(0xFFFFFFFFu, o, 0) + __popc(mids & ((1u << lane) - 1u));
+      if (kind == 3) {
+        if (o < lcap) {
+          float4* d = reinterpret_cast<float4*>(A.cand + lbase + o);
+          d[0] = make_float4(__int_as_float(E.v.X[0]), __int_as_float(E.v.Y[0]), __int_as_float(E.v.X[1]),
+                             __int_as_float(E.v.Y[1]));
+          d[1] = make_float4(__int_as_float(E.v.X[2]), __int_as_float(E.v.Y[2]),
+                             __int_as_float(E.px0 | (E.py0 << 16)), __int_as_float(E.px1 | (E.py1 << 16)));
+          d[2] = make_float4(E.v.z[0], E.v.z[1], E.v.z[2], __uint_as_float(t));
+        } else {
+          win_box<4>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
+        }
+      }
+    }
+    // large triangles of the warp reserve queue records and tiles with one atomic
+    const uint32_t bigs = __ballot_sync(0xFFFFFFFFu, kind == 2);
+    if (bigs) {
+      uint32_t tpre = tiles;  // inclusive prefix of tiles over the warp
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, tpre, o);
+        if (lane >= (unsigned)o) tpre += y;
+      }
+      const uint32_t ttot = __shfl_sync(0xFFFFFFFFu, tpre, 31);
+      unsigned long long old = 0;
+      if (lane == 0)
+        old = atomicAdd(&A.ctr->big, ((unsigned long long)__popc(bigs) << 40) | (unsigned long long)ttot);
+      old = __shfl_sync(0xFFFFFFFFu, old, 0);
+      if (kind == 2 &&
+          !win_queue(A, E.v.X, E.v.Y, E.v.z, E.px0, E.py0, E.px1, E.py1, E.fits, t,
+                     (old >> 40) + __popc(bigs & ((1u << lane) - 1u)), (old & ((1ull << 40) - 1)) + (tpre - tiles), tiles)) {
+        const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
+        win_rect64<false>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
+      }
+    }
+    if (!grouped) {
+      if (kind == 1) win_box<4>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
+    } else {
+      // the group's leader holds the triangle; each lane takes one sample of its box
+      const uint32_t src = lane & ~(kRasterGroup - 1u);
+      Tri32 g;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        g.X[j] = __shfl_sync(0xFFFFFFFFu, E.v.X[j], src);
+        g.Y[j] = __shfl_sync(0xFFFFFFFFu, E.v.Y[j], src);
+        g.z[j] = __shfl_sync(0xFFFFFFFFu, E.v.z[j], src);
+      }
+      const int px0 = __shfl_sync(0xFFFFFFFFu, E.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, E.py0, src);
+      const int px1 = __shfl_sync(0xFFFFFFFFu, E.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, E.py1, src);
+      const uint32_t gt = __shfl_sync(0xFFFFFFFFu, t, src);
+      const bool go = __shfl_sync(0xFFFFFFFFu, kind, src) == 1;
+      if (go) win_box<1>(A, g, gt, px0, py0, px1, py1, (int)sub, (int)kRasterGroup);
+    }
+  }
+  // then the (rare) triangles that need clipping, from the front blocks' regions
+  __syncthreads();  // pre is reused
+  const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
+  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
+    const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
+    const uint32_t* f = A.idx + 3 * (size_t)t;
+    const Mat4 M = DEV_M ? load_mat(A.Mdev) : A.M;
+    win_clipped<false>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
+                       load_clip(M, A.pos, __ldg(f + 2)));
+  }
+}
+
+// The queued tiles, a warp each, then the mid-size lists.
+__device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  __shared__ uint32_t pre[kMidLists + 1];
+  const uint32_t lane = threadIdx.x & 31;
+  __syncthreads();  // pre of an earlier item of the same block is free
+  if (threadIdx.x < 32) {
+    uint32_t c = 0;
+    if (lane < A.mid_lists) c = min(__ldcg(&A.ctr->n_mid[lane][0]), mid_base(A, lane + 1u) - mid_base(A, lane));
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= (unsigned)o) x += y;
+    }
+    pre[lane + 1] = x;
+    if (lane == 0) pre[0] = 0u;
+  }
+  const uint32_t warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = (nblk * blockDim.x) >> 5;
+  const unsigned long long st = __ldcg(&A.ctr->big);
+  const uint32_t n_ent = (uint32_t)min((unsigned long long)A.queue_cap, st >> 40);
+  const uint32_t n_tiles = n_ent ? (uint32_t)min((unsigned long long)A.tile_cap, st & ((1ull << 40) - 1)) : 0u;
+  for (uint32_t g = warp; g < n_tiles; g += nwarps) {
+    const uint32_t lo = __ldcg(A.tile_owner + g);
+    if (lo >= n_ent) continue;
+    const BigTri& q = A.queue[lo];
+    const int px0 = q.px0, py0 = q.py0, px1 = q.px1, py1 = q.py1;
+    if (px1 < px0 || py1 < py0) continue;
+    const uint32_t tx_n = (uint32_t)((px1 - px0 + kBigTile) / kBigTile);
+    const uint32_t local = g - q.tile0;
+    const int bx = px0 + (int)(local % tx_n) * kBigTile, by = py0 + (int)(local / tx_n) * kBigTile;
+    if (by > py1) continue;
+    const uint32_t t = q.tri;
+    const int px = bx + (int)(lane % kBigTile), py_first = by + (int)(lane / kBigTile);
+    const int py_last = min(by + kBigTile - 1, py1);
+    Put put;
+    if (q.pad) {
+      const Tri32 v{{q.X[0], q.X[1], q.X[2]}, {q.Y[0], q.Y[1], q.Y[2]}, {q.zn[0], q.zn[1], q.zn[2]}};
+      const Edges32 E = edges32(v, px, py_first);
+      int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2];
+      PutN<4> q4;
+      if (px <= px1)
+        for (int py = py_first; py <= py_last;) {
+          uint32_t key[4], pix[4];
+          bool on[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            pix[i] = (uint32_t)py * (uint32_t)A.W + (uint32_t)px;
+            on[i] = (e0 | e1 | e2) >= 0 && py <= py_last && key32(E, e0, e1, e2, v, key[i]);
+            e0 += E.dy[0] * (32 / kBigTile);
+            e1 += E.dy[1] * (32 / kBigTile);
+            e2 += E.dy[2] * (32 / kBigTile);
+            py += 32 / kBigTile;
+          }
+          q4.put(A, t, on, key, pix);
+        }
+      q4.check(A, t);
+    } else {
+      const SV a{q.X[0], q.Y[0], q.zn[0]}, b{q.X[1], q.Y[1], q.zn[1]}, c{q.X[2], q.Y[2], q.zn[2]};
+      const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
+      const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
+      const Edges E = edges_at(a, b, c, px, py_first);
+      int64_t e[3] = {E.e[0], E.e[1], E.e[2]};
+      if (px <= px1)
+#pragma unroll 1
+        for (int py = py_first; py <= py_last; py += 32 / kBigTile) {
+          const bool in = (e[0] > 0 || (e[0] == 0 && E.tl[0])) && (e[1] > 0 || (e[1] == 0 && E.tl[1])) &&
+                          (e[2] > 0 || (e[2] == 0 && E.tl[2]));
+          if (in) {
+            float s = __fmul_rn(ll2float_rn(e[0]), a.zn);
+            s = __fadd_rn(s, __fmul_rn(ll2float_rn(e[1]), b.zn));
+            s = __fadd_rn(s, __fmul_rn(ll2float_rn(e[2]), c.zn));
+            const float d = __fmul_rn(s, invA);
+            if (d >= -1.0f && d <= 1.0f) {
+              put.put(A, (uint32_t)py * (uint32_t)A.W + (uint32_t)px, ordered(d), t);
+            }
+          }
+          e[0] += E.dy[0] * (32 / kBigTile);
+          e[1] += E.dy[1] * (32 / kBigTile);
+          e[2] += E.dy[2] * (32 / kBigTile);
+        }
+    }
+    put.check(A, t);
+  }
+  __syncthreads();
+  const uint32_t n = pre[kMidLists], stride = nblk * blockDim.x;
+  uint32_t lg = kMinLanes;
+  while (lg < 5u && ((uint64_t)n << (lg + 1u)) <= stride) ++lg;
+  const uint32_t sub = threadIdx.x & ((1u << lg) - 1u);
+  for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> lg; i < n; i += stride >> lg) {
+    uint32_t lo = 0, hi = kMidLists;  // pre[lo] <= i < pre[hi]
+    while (hi - lo > 1u) {
+      const uint32_t mid = (lo + hi) >> 1;
+      if (pre[mid] <= i) lo = mid;
+      else hi = mid;
+    }
+    const float4* s = reinterpret_cast<const float4*>(A.cand + mid_base(A, lo) + (i - pre[lo]));
+    const float4 f0 = __ldcs(s), f1 = __ldcs(s + 1), f2 = __ldcs(s + 2);
+    const Tri32 v{{__float_as_int(f0.x), __float_as_int(f0.z), __float_as_int(f1.x)},
+                  {__float_as_int(f0.y), __float_as_int(f0.w), __float_as_int(f1.y)},
+                  {f2.x, f2.y, f2.z}};
+    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
+    win_box<4>(A, v, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu), (int)(b1 >> 16),
+               (int)sub, 1 << lg);
+  }
+}
+
+// Sets triangle t's visible bit.
+__device__ __forceinline__ void win_mark(const RasterArgs& A, uint32_t t) {
+  const uint32_t bit = 1u << (t & 31);
+  if (__ldcg(A.vt + (t >> 5)) & bit) return;
+  atomicOr(A.vt + (t >> 5), bit);
+  note_tile(A, t >> 10);
+}
+
+// The marking pass when the tie list overflowed: every survivor and clipped triangle
+// tested against the final keys.
+template <int NT>
+__device__ __noinline__ void mark_all(const RasterArgs& A, uint32_t bid, uint32_t nblk, uint32_t* pre) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t n = surv_prefix<NT>(A, pre);
+  const uint32_t stride = nblk * blockDim.x;
+  for (uint32_t wbase = bid * blockDim.x + (threadIdx.x & ~31u); wbase < n; wbase += stride) {
+    const uint32_t v = wbase + lane;
+    WinSetup E = {};
+    uint32_t t = 0;
+    bool vis = false, large = false;
+    if (v < n) {
+      const uint32_t i = surv_slot(A, pre, v, wbase);
+      const float4* sc = A.surv_clip + 3 * (size_t)i;
+      t = __ldcg(A.surv + i);
+      E = win_setup(A, sc[0], sc[1], sc[2]);
+      if (E.live) {
+        large = (E.px1 - E.px0 + 1) * (E.py1 - E.py0 + 1) > kMidPix;
+        const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
+        if (!large) vis = win_rect64<true>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
+      }
+    }
+    for (uint32_t m = __ballot_sync(0xFFFFFFFFu, large); m; m &= m - 1u) {  // the warp together
+      const int src = __ffs(m) - 1;
+      SV q[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        q[j] = SV{__shfl_sync(0xFFFFFFFFu, E.v.X[j], src), __shfl_sync(0xFFFFFFFFu, E.v.Y[j], src),
+                  __shfl_sync(0xFFFFFFFFu, E.v.z[j], src)};
+      const int px0 = __shfl_sync(0xFFFFFFFFu, E.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, E.py0, src);
+      const int px1 = __shfl_sync(0xFFFFFFFFu, E.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, E.py1, src);
+      const bool hit = win_rect64<true>(A, q[0], q[1], q[2], 0u, px0, py0, px1, py1, lane, 32u);
+      if (__any_sync(0xFFFFFFFFu, hit) && (int)lane == src) vis = true;
+    }
+    if (vis) win_mark(A, t);
+  }
+  __syncthreads();  // pre is reused
+  const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
+  const Mat4 M = A.Mdev ? load_mat(A.Mdev) : A.M;
+  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
+    const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
+    const uint32_t* f = A.idx + 3 * (size_t)t;
+    if (win_clipped<true>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
+                          load_clip(M, A.pos, __ldg(f + 2))))
+      win_mark(A, t);
+  }
+}
+
+// Marking: the triangle of every pixel, then the listed ties whose key is the pixel's.
+template <int NT>
+__device__ __forceinline__ void mark_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  uint32_t* pre = region_pre();
+  __shared__ int32_t s_status;
+  __shared__ uint32_t s_ties;
+  __syncthreads();  // the shared words of an earlier item of the same block are free
+  if (threadIdx.x == 0) {
+    s_status = __ldcg(&A.ctr->status);
+    s_ties = __ldcg(&A.ctr->n_ties);
+  }
+  __syncthreads();
+  if (s_status != 0) return;
+  // A warp takes 64 x kR pixels, two side by side a thread in each row, the block's warps
+  // one below the other.  A pixel whose left or upper neighbour has the same triangle is
+  // passed over; what is left is looked up in a table of the triangles (and the tiles) the
+  // block marked last, so that a triangle costs one atomic for all its pixels in a block.
+  constexpr uint32_t kNone = 0xFFFFFFFFu;
+  constexpr uint32_t kR = 4, kSeen = 1024, kSeenTiles = 64;
+  __shared__ uint32_t seen[kSeen], seen_tile[kSeenTiles];
+  for (uint32_t i = threadIdx.x; i < kSeen; i += blockDim.x) seen[i] = kNone;
+  if (threadIdx.x < kSeenTiles) seen_tile[threadIdx.x] = kNone;
+  __syncthreads();
+  volatile uint32_t* vseen = seen;
+  volatile uint32_t* vtile = seen_tile;
+  const uint32_t lane = threadIdx.x & 31;
+  constexpr uint32_t kRows = kR * (NT / 32);
+  const uint32_t cols = ((uint32_t)A.W + 63u) / 64u, bands = ((uint32_t)A.H + kRows - 1u) / kRows;
+  for (uint32_t g = bid; g < cols * bands; g += nblk) {
+    const uint32_t x = (g % cols) * 64u + 2u * lane, y0 = (g / cols) * kRows + (threadIdx.x >> 5) * kR;
+    uint2 q[2 * kR];  // (triangle, key)
+#pragma unroll
+    for (uint32_t r = 0; r < kR; ++r) {
+      const uint2* z = reinterpret_cast<const uint2*>(A.zid) + (size_t)(y0 + r) * A.W + x;
+      const bool row = y0 + r < (uint32_t)A.H;
+      q[2 * r] = row && x < (uint32_t)A.W ? __ldcg(z) : make_uint2(kNone, kNone);
+      q[2 * r + 1] = row && x + 1u < (uint32_t)A.W ? __ldcg(z + 1) : make_uint2(kNone, kNone);
+    }
+    uint32_t t[2 * kR];
+#pragma unroll
+    for (uint32_t r = 0; r < kR; ++r) {
+      const uint32_t a = q[2 * r].y != kNone ? q[2 * r].x : kNone, b = q[2 * r + 1].y != kNone ? q[2 * r + 1].x : kNone;
+      const uint32_t up_a = r && q[2 * r - 2].y != kNone ? q[2 * r - 2].x : kNone;
+      const uint32_t up_b = r && q[2 * r - 1].y != kNone ? q[2 * r - 1].x : kNone;
+      const uint32_t left = __shfl_up_sync(0xFFFFFFFFu, b, 1);
+      t[2 * r] = (lane && left == a) || up_a == a ? kNone : a;
+      t[2 * r + 1] = b == a || up_b == b ? kNone : b;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < 2 * kR; ++u) {
+      const uint32_t m = t[u];
+      if (m == kNone || vseen[m % kSeen] == m) continue;
+      vseen[m % kSeen] = m;
+      atomicOr(A.vt + (m >> 5), 1u << (m & 31));
+      const uint32_t tile = m >> 10;
+      if (vtile[tile % kSeenTiles] == tile) continue;
+      vtile[tile % kSeenTiles] = tile;
+      note_tile(A, tile);
+    }
+  }
+  const uint32_t stride = nblk * blockDim.x;
+  if (s_ties <= A.tie_cap) {
+    for (uint32_t i = bid * blockDim.x + threadIdx.x; i < s_ties; i += stride) {
+      const uint4 e = __ldcg(A.ties + i);
+      if (zkey(A, e.x) == e.y) {
+        win_mark(A, e.z);
+        win_mark(A, e.w);
+      }
+    }
+  } else {
+    mark_all<NT>(A, bid, nblk, pre);
+  }
+}
+
+inline void set_raster_mode(RasterArgs& A);
+
 // The arguments of one visibility pass on ctx (host side).  front_blocks blocks of
 // `threads` threads run the front end; each owns a survivor region large enough for
 // every triangle it can see.
@@ -1103,7 +1774,23 @@ inline RasterArgs make_raster_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4&
   A.clip = ctx->clip;
   A.ctr = ctx->ctr;
   A.vt = vt;
+  A.zid = reinterpret_cast<unsigned long long*>(ctx->zbuf);
+  A.ties = ctx->ties;
+  A.tie_cap = ctx->tie_cap;
+  set_raster_mode(A);
   return A;
+}
+
+// Conservative marking tests other samples than the depth pass takes, and the tile-depth
+// option belongs to the second rasterization: both keep it.
+inline void set_raster_mode(RasterArgs& A) { A.win = !A.cons && !A.zmax ? 1 : 0; }
+
+// The exact pass's grid (blocks of `threads` threads), from which the mid-size lists get
+// their shares: a block sees at most mid_per_block survivors.
+inline void set_exact_grid(RasterArgs& A, uint32_t blocks, uint32_t threads) {
+  A.mid_blocks = blocks;
+  A.mid_lists = blocks < (uint32_t)kMidLists ? blocks : (uint32_t)kMidLists;
+  A.mid_per_block = (uint32_t)(((uint64_t)A.T + (uint64_t)blocks * threads - 1) / ((uint64_t)blocks * threads)) * threads;
 }
 
 }  // namespace
