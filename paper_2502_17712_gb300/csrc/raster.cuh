@@ -1095,15 +1095,17 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
 // ones do.  A top-left edge passes at 0, another one from 1, so that with 1 taken from
 // the others a sample is covered when no value is negative.
 //
-// What bounds it: the atomics' round trips and, on views of many mid-size triangles,
-// their issue (about 120 G samples/s).  Four samples of a lane are on their way at once
-// (one: 851 us for the larger boxes of a 3.2M-triangle floor at 1440p; four: 379;
-// eight spill: 999) and at least four lanes share a box, so that their atomics meet in
-// a sector (one lane: 446 us, two 384, four 374, eight 420).  A load of the pixel's key
-// before the atomic costs more than the atomics it saves (471 us).  Against two
-// rasterizations, exact + larger boxes + marking: that floor 2475 -> 551 us, a floor of
-// 60 patches at 1080p 247 -> 89, 200 icospheres at 1080p 107 -> 63, one patch of
-// 7,938 triangles at 1080p 52 -> 43 (events around each kernel, GB300).
+// What bounds it: the atomics' round trips and the instructions of the samples (the
+// larger boxes of a 3.2M-triangle floor at 1440p issue 60 % of the cycles).  Times of
+// that pass: one sample of a lane at a time 851 us; four at once, their returned values
+// looked at after the next four, 317 (three 332; six 447; looked at at once 485, which
+// is the better way only for the small boxes' four rounds at most, 125 against 160).
+// At least four lanes share a box, so that their atomics meet in a sector (one lane
+// 446 us, two 384, four 374, eight 420, at three blocks per SM).  A load of the pixel's
+// key before the atomic costs more than the atomics it saves (471 us against 379).
+// Against two rasterizations, exact + larger boxes + marking: that floor 2475 -> 459
+// us, 60 patches at 1080p 247 -> 83, 200 icospheres at 1080p 107 -> 62, one patch of
+// 7,938 triangles at 1080p 52 -> 40 (events around each kernel, GB300).
 constexpr int kMidPix = 256;  // (512: the same)
 constexpr uint32_t kMinLanes = 2;  // log2 of the fewest lanes a mid-size box gets
 constexpr int kSpan32 = 96 * kSub;  // side of a sub-triangle with 32-bit edge functions
@@ -1198,17 +1200,35 @@ __device__ __forceinline__ bool key32(const Edges32& E, int e0, int e1, int e2, 
   float s = __fmul_rn(__int2float_rn(e0 + E.nb[0]), v.z[0]);
   s = __fadd_rn(s, __fmul_rn(__int2float_rn(e1 + E.nb[1]), v.z[1]));
   s = __fadd_rn(s, __fmul_rn(__int2float_rn(e2 + E.nb[2]), v.z[2]));
-  const float d = __fmul_rn(s, E.invA);
-  key = ordered(d);
-  return d >= -1.0f && d <= 1.0f;
+  const float d = __fadd_rn(__fmul_rn(s, E.invA), 0.0f);  // (-0 becomes +0)
+  const uint32_t u = __float_as_uint(d);
+  key = u ^ ((uint32_t)((int32_t)u >> 31) | 0x80000000u);  // ordered(d)
+  return fabsf(d) <= 1.0f;
 }
 
 __device__ __forceinline__ uint32_t zkey(const RasterArgs& A, uint32_t pix) {
   return __ldcg(reinterpret_cast<const uint32_t*>(A.zid) + 2 * (size_t)pix + 1);
 }
 
-// A thread's N samples on their way: keys put, and the old values of the N before them,
-// which are looked at once these are issued.
+// Puts a thread's N samples (those that are on): their atomics are all on their way
+// before the first returned value is looked at.
+template <int N>
+__device__ __forceinline__ void put_n(const RasterArgs& A, uint32_t t, const bool (&on)[N], const uint32_t (&key)[N],
+                                      const uint32_t (&pix)[N]) {
+  unsigned long long old[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    old[i] = ~0ull;
+    if (on[i]) old[i] = atomicMin(A.zid + pix[i], ((unsigned long long)key[i] << 32) | t);
+  }
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (on[i] && (uint32_t)(old[i] >> 32) == key[i] && (uint32_t)old[i] != t)
+      note_tie(A, pix[i], key[i], (uint32_t)old[i], t);
+}
+
+// The same with the returned values looked at only when the thread's next N are on their
+// way (or at the end): for loops of many rounds, where each would wait for its own.
 template <int N>
 struct PutN {
   unsigned long long old[N];
@@ -1229,8 +1249,10 @@ struct PutN {
                                       const uint32_t (&p)[N]) {
     unsigned long long o[N];
 #pragma unroll
-    for (int i = 0; i < N; ++i)
-      o[i] = on[i] ? atomicMin(A.zid + p[i], ((unsigned long long)k[i] << 32) | t) : ~0ull;
+    for (int i = 0; i < N; ++i) {
+      o[i] = ~0ull;
+      if (on[i]) o[i] = atomicMin(A.zid + p[i], ((unsigned long long)k[i] << 32) | t);
+    }
     check(A, t);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
@@ -1243,7 +1265,7 @@ struct PutN {
 
 // Samples first, first + step, .. (row order) of a 32-bit sub-triangle's box, N at a time
 // so that their atomics overlap.  step lanes side by side then put neighbouring pixels.
-template <int N>
+template <int N, bool LATER = false>
 __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uint32_t t, int px0, int py0, int px1,
                                         int py1, int first, int step) {
   const int w = px1 - px0 + 1, n = w * (py1 - py0 + 1);
@@ -1257,14 +1279,14 @@ __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uin
   const uint32_t ap = (uint32_t)(A.W * sy + sx), bp = ap + (uint32_t)(A.W - w);
   int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2], col = w - fx;  // col: pixels to the row's end
   uint32_t p = (uint32_t)(py0 + fy) * (uint32_t)A.W + (uint32_t)(px0 + fx);
-  PutN<N> q;
-  for (int s = first; s < n;) {
+  PutN<LATER ? N : 1> later;
+  for (int left = n - 1 - first; left >= 0;) {  // (negative once the box is done)
     uint32_t key[N], pix[N];
     bool on[N];
 #pragma unroll
     for (int i = 0; i < N; ++i) {
       pix[i] = p;
-      on[i] = (e0 | e1 | e2) >= 0 && s < n && key32(E, e0, e1, e2, v, key[i]);
+      on[i] = (e0 | e1 | e2 | left) >= 0 && key32(E, e0, e1, e2, v, key[i]);
       col -= sx;
       const bool wrap = col <= 0;
       col += wrap ? w : 0;
@@ -1272,11 +1294,12 @@ __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uin
       e1 += wrap ? b1 : a1;
       e2 += wrap ? b2 : a2;
       p += wrap ? bp : ap;
-      s += step;
+      left -= step;
     }
-    q.put(A, t, on, key, pix);
+    if constexpr (LATER) later.put(A, t, on, key, pix);
+    else put_n(A, t, on, key, pix);
   }
-  q.check(A, t);
+  if constexpr (LATER) later.check(A, t);
 }
 
 // Any sub-triangle, 64-bit edge functions: samples first, first + step, .. of its box in
@@ -1526,7 +1549,7 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
       const Tri32 v{{q.X[0], q.X[1], q.X[2]}, {q.Y[0], q.Y[1], q.Y[2]}, {q.zn[0], q.zn[1], q.zn[2]}};
       const Edges32 E = edges32(v, px, py_first);
       int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2];
-      PutN<4> q4;
+      PutN<4> later;
       if (px <= px1)
         for (int py = py_first; py <= py_last;) {
           uint32_t key[4], pix[4];
@@ -1540,9 +1563,9 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
             e2 += E.dy[2] * (32 / kBigTile);
             py += 32 / kBigTile;
           }
-          q4.put(A, t, on, key, pix);
+          later.put(A, t, on, key, pix);
         }
-      q4.check(A, t);
+      later.check(A, t);
     } else {
       const SV a{q.X[0], q.Y[0], q.zn[0]}, b{q.X[1], q.Y[1], q.zn[1]}, c{q.X[2], q.Y[2], q.zn[2]};
       const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
@@ -1588,7 +1611,7 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
                   {__float_as_int(f0.y), __float_as_int(f0.w), __float_as_int(f1.y)},
                   {f2.x, f2.y, f2.z}};
     const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
-    win_box<4>(A, v, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu), (int)(b1 >> 16),
+    win_box<4, true>(A, v, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu), (int)(b1 >> 16),
                (int)sub, 1 << lg);
   }
 }
