@@ -243,6 +243,7 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(const __grid_constant__ Pers
   // the loop keeps nothing in registers across a stage body (every value is re-read
   // from shared memory or the parameter), so that a body has the whole budget
   __shared__ uint32_t s_item, s_g, s_skip;
+  if (threadIdx.x == 0) s_g = 0u;
   for (;;) {
     if (threadIdx.x == 0) {
       const Group* groups = SINGLE ? P.inline_groups : P.groups;
@@ -250,13 +251,10 @@ __global__ void __launch_bounds__(kPT, 1) k_persist(const __grid_constant__ Pers
       const uint32_t item = atomicAdd(P.sched, 1u);
       uint32_t g = 0, skip = 1;
       if (item < P.n_items) {
-        uint32_t lo = 0, hi = P.n_groups;  // the last group starting at or before item
-        while (hi - lo > 1) {
-          const uint32_t mid = (lo + hi) >> 1;
-          if (groups[mid].start <= item) lo = mid;
-          else hi = mid;
-        }
-        g = lo;
+        // the last group starting at or before item: this CTA's claims only grow, so
+        // from the group of its last one (mostly the same or the next)
+        g = s_g;
+        while (g + 1u < P.n_groups && groups[g + 1u].start <= item) ++g;
         const int32_t dep = groups[g].dep;
         skip = ld_acquire(abort) ? 1u : 0u;
         if (!skip && dep >= 0)
