@@ -256,8 +256,6 @@ fa_status fa_chartify(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* d_vt, ui
   return st;
 }
 
-// The box and UV kernels walk the context's visible-triangle list; the standalone
-// calls build it from tri_chart so that they need no extra argument.
 fa_status fa_parameterize(fa_ctx* ctx, const fa_mesh* mesh, const float view_proj[16], uint32_t width,
                           uint32_t height, float ratio, const int32_t* d_tri_chart, const fa_charts* charts,
                           uint32_t flags, uint32_t* d_partial, fa_stream_t stream) {
@@ -270,10 +268,8 @@ fa_status fa_parameterize(fa_ctx* ctx, const fa_mesh* mesh, const float view_pro
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   trace_begin(ctx);
-  st = launch_vis_list(ctx, mesh, d_tri_chart, s);
-  if (st == FA_OK)
-    st = launch_parameterize(ctx, mesh, to_mat(view_proj), width, height, ratio, d_tri_chart, charts, true, flags,
-                             d_partial, s);
+  st = launch_parameterize(ctx, mesh, to_mat(view_proj), width, height, ratio, d_tri_chart, charts, true, flags,
+                           d_partial, s, nullptr, true, false);
   trace_end(ctx, s);
   return st;
 }
@@ -306,10 +302,8 @@ fa_status fa_uv(fa_ctx* ctx, const fa_mesh* mesh, const float view_proj[16], uin
   DeviceGuard g(ctx->device);
   cudaStream_t s = (cudaStream_t)stream;
   trace_begin(ctx);
-  st = launch_vis_list(ctx, mesh, d_tri_chart, s);
-  if (st == FA_OK)
-    st = launch_uv(ctx, mesh, to_mat(view_proj), width, height, ratio, d_tri_chart, charts, d_place, d_res,
-                   atlas_log2, n_scales, d_uv, d_affine, s);
+  st = launch_uv(ctx, mesh, to_mat(view_proj), width, height, ratio, d_tri_chart, charts, d_place, d_res,
+                 atlas_log2, n_scales, d_uv, d_affine, s, nullptr, false, false);
   trace_end(ctx, s);
   return st;
 }

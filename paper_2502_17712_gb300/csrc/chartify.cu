@@ -1,6 +1,5 @@
 // Chart kernels (Sec. 5.1; App. A "GPU Union Find", Alg. 1): the launch wrappers
-// of the stage bodies in chartify.cuh, the standalone visible-list kernels and the
-// launch sequence of one chart pass.
+// of the stage bodies in chartify.cuh and the launch sequence of one chart pass.
 #include <algorithm>
 
 #include "chartify.cuh"
@@ -67,11 +66,6 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(uint32_t* blockcnt, uint32
   cf::scan_blocks_body(blockcnt, viscnt, nblocks, count_out, max_charts, ctr);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_vis(uint32_t* viscnt, uint32_t nblocks, DevCounters* ctr) {
-  pdl_wait();
-  cf::scan_vis_body(viscnt, nblocks, ctr);
-}
-
 template <bool LIST>
 __global__ void __launch_bounds__(kBlock) k_tri_chart(UfArgs a, const uint32_t* blockcnt, const uint2* wordroots,
                                                       int32_t* tri_chart, uint32_t* roots, uint32_t* box_enc,
@@ -86,42 +80,6 @@ __global__ void k_vert_chart(UfArgs a, const uint32_t* blockcnt, const uint2* wo
                              int vertex_mode) {
   pdl_wait();
   cf::vert_chart_body(a, blockcnt, wordroots, vert_chart, vertex_mode, blockIdx.x, gridDim.x);
-}
-
-// Standalone path: visible counts per block from a caller's tri_chart ...
-__global__ void __launch_bounds__(kBlock) k_vis_count(const int32_t* tri_chart, uint32_t T, uint32_t* viscnt) {
-  pdl_wait();
-  __shared__ uint32_t vc[kBlock / 32];
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t v = 0;
-#pragma unroll
-  for (uint32_t k = 0; k < kPerBlock / kBlock; ++k) {
-    const uint32_t t = blockIdx.x * kPerBlock + (k * (kBlock / 32) + wid) * 32 + lane;
-    v += __popc(__ballot_sync(0xFFFFFFFFu, t < T && tri_chart[t] >= 0));
-  }
-  if (lane == 0) vc[wid] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    uint32_t s = 0;
-    for (int i = 0; i < kBlock / 32; ++i) s += vc[i];
-    viscnt[blockIdx.x] = s;
-  }
-}
-
-// ... and the list itself, after k_scan_vis.
-__global__ void __launch_bounds__(kBlock) k_vis_fill(const int32_t* tri_chart, uint32_t T, const uint32_t* visstart,
-                                                     uint2* vis) {
-  pdl_wait();
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t words[kPerBlock / kBlock];
-  int32_t chart[kPerBlock / kBlock];
-#pragma unroll
-  for (uint32_t k = 0; k < kPerBlock / kBlock; ++k) {
-    const uint32_t t = blockIdx.x * kPerBlock + (k * (kBlock / 32) + wid) * 32 + lane;
-    chart[k] = t < T ? tri_chart[t] : -1;
-    words[k] = __ballot_sync(0xFFFFFFFFu, chart[k] >= 0);
-  }
-  cf::put_visible<kBlock>(words, __ldcg(visstart + blockIdx.x), chart, vis, blockIdx.x);
 }
 
 }  // namespace
@@ -176,18 +134,6 @@ fa_status launch_chartify(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* vt, 
     launch_k(k_vert_chart, grid_for(mesh->V, 256, 152 * 8), 256, 0, s, a, ctx->blockcnt, ctx->wordroots,
              vert_chart, vm);
   }
-  FA_CUDA_TRY(cudaGetLastError());
-  return FA_OK;
-}
-
-fa_status launch_vis_list(fa_ctx* ctx, const fa_mesh* mesh, const int32_t* tri_chart, cudaStream_t s) {
-  const uint32_t nb = (mesh->T + kPerBlock - 1) / kPerBlock;
-  mark(ctx, "k_vis_count", s);
-  launch_k(k_vis_count, nb ? nb : 1, kBlock, 0, s, tri_chart, mesh->T, ctx->viscnt);
-  mark(ctx, "k_scan_vis", s);
-  launch_k(k_scan_vis, 1, 1024, 0, s, ctx->viscnt, nb ? nb : 1, ctx->ctr);
-  mark(ctx, "k_vis_fill", s);
-  launch_k(k_vis_fill, nb ? nb : 1, kBlock, 0, s, tri_chart, mesh->T, ctx->viscnt, ctx->vis);
   FA_CUDA_TRY(cudaGetLastError());
   return FA_OK;
 }

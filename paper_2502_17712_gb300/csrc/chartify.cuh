@@ -209,6 +209,13 @@ __device__ __forceinline__ void local_tile(const UfArgs& a, uint32_t tile) {
   if (threadIdx.x == 0) a.xcnt[tile] = s_xc;  // all appends precede the last barrier
 }
 
+// Entry i of the tile list, or anything past its room: read before the list's length is
+// known, so that the two loads do not wait for one another (a frame's kernels are chains
+// of such loads, about 0.4 us each).
+__device__ __forceinline__ uint32_t list_entry(const UfArgs& a, uint32_t i) {
+  return i < (a.T + kTile - 1) / kTile ? __ldcg(a.tile_list + i) : 0u;
+}
+
 // Every tile (a block each), or only the tiles that the marking pass listed (a
 // persistent grid over the list).
 template <bool LIST, int NT>
@@ -224,10 +231,11 @@ __device__ __forceinline__ void local_body(const UfArgs& a, uint32_t bid, uint32
   // the first tile by block index, the others handed out by a counter, so that a
   // block that drew light tiles takes more (their costs differ by an order of
   // magnitude) and the blocks do not all queue on the counter at once
-  const uint32_t n = __ldcg(&a.ctr->n_vtiles);
+  // (the count and the first entry, which may be left from an earlier frame, at once)
+  const uint32_t n = __ldcg(&a.ctr->n_vtiles), first = list_entry(a, bid);
   __shared__ uint32_t s_i;
   for (uint32_t i = bid; i < n;) {
-    local_tile<NT>(a, __ldcg(a.tile_list + i));
+    local_tile<NT>(a, i == bid ? first : __ldcg(a.tile_list + i));
     __syncthreads();  // the shared memory of this tile is free, and s_i was read
     if (threadIdx.x == 0) s_i = nblk + atomicAdd(&a.ctr->uf_item, 1u);
     __syncthreads();
@@ -246,10 +254,11 @@ __device__ __forceinline__ void init_v_body(int32_t* label, uint32_t T, uint32_t
 // t0 / nt: this thread's index in the group of threads that hooks the tile, and the
 // group's size (the block, or a slice of it).
 __device__ __forceinline__ void hook_tile(const UfArgs& a, uint32_t tile, uint32_t t0, uint32_t nt) {
-  const uint32_t n = min(__ldcg(a.xcnt + tile), kXCap);
   const uint2* xe = a.xedge + (size_t)tile * kXCap;
+  uint2 e = __ldcg(xe + t0);  // (with the count; t0 < kXCap)
+  const uint32_t n = min(__ldcg(a.xcnt + tile), kXCap);
   for (uint32_t i = t0; i < n; i += nt) {
-    const uint2 e = __ldcg(xe + i);
+    if (i != t0) e = __ldcg(xe + i);
     if (e.y < a.T && vt_bit(a.vt, e.y)) unite(a.label, (int32_t)e.x, (int32_t)e.y, a.ctr, a.loop_cap);
   }
 }
@@ -265,8 +274,13 @@ __device__ __forceinline__ void hook_body(const UfArgs& a, uint32_t bid, uint32_
     for (uint32_t t = grp; t < ntiles; t += ngrp) hook_tile(a, t, t0, gt);
     return;
   }
+  uint32_t next = list_entry(a, grp);
   const uint32_t n = __ldcg(&a.ctr->n_vtiles);
-  for (uint32_t i = grp; i < n; i += ngrp) hook_tile(a, __ldcg(a.tile_list + i), t0, gt);
+  for (uint32_t i = grp; i < n; i += ngrp) {
+    const uint32_t tile = next;
+    next = list_entry(a, i + ngrp);
+    hook_tile(a, tile, t0, gt);
+  }
 }
 
 // Vertex mode: every visible triangle joins its three vertex nodes T + v.
@@ -495,11 +509,6 @@ __device__ __forceinline__ void scan_blocks_body(uint32_t* blockcnt, uint32_t* v
   }
 }
 
-// Scan of the visible counts alone (the standalone box / UV calls).
-__device__ __forceinline__ void scan_vis_body(uint32_t* viscnt, uint32_t nblocks, DevCounters* ctr) {
-  scan_counts(viscnt, nullptr, nblocks, &ctr->n_vis, nullptr);
-}
-
 // The entries of one 1024-triangle block's visible triangles in the list, in
 // triangle order: entry = list start of the block + the visible triangles before
 // it.  words[k] is VT word k * (NT / 32) + warp of the block.
@@ -547,18 +556,15 @@ __device__ __forceinline__ void chart_tile(const UfArgs& a, uint32_t tile, const
   constexpr uint32_t kK = kPerBlock / NT;
   uint32_t words[kK], rt[kK];
   int32_t chart[kK];
-  // the loads of the thread's kK triangles in rounds (VT words, roots, the roots'
+  // the loads of the thread's kK triangles in rounds (VT words and roots, the roots'
   // counts), each round independent, before any store
 #pragma unroll
   for (uint32_t k = 0; k < kK; ++k) {
-    const uint32_t w = tile * (kPerBlock / 32) + k * (NT / 32) + wid;
+    const uint32_t w = tile * (kPerBlock / 32) + k * (NT / 32) + wid, t = (w << 5) + lane;
     words[k] = w < nwords ? __ldcg(a.vt + w) : 0u;
+    rt[k] = t < a.T ? (uint32_t)__ldcg(a.label + t) : 0u;  // (with the word: any value where not visible)
   }
-#pragma unroll
-  for (uint32_t k = 0; k < kK; ++k) {
-    const uint32_t t = ((tile * (kPerBlock / 32) + k * (NT / 32) + wid) << 5) + lane;
-    rt[k] = (words[k] >> lane) & 1u ? (uint32_t)__ldcg(a.label + t) : 0u;
-  }
+  const uint32_t start = __ldcg(visstart + tile);
 #pragma unroll
   for (uint32_t k = 0; k < kK; ++k)
     chart[k] = (words[k] >> lane) & 1u ? (int32_t)chart_of_root(blockcnt, wordroots, rt[k]) : -1;
@@ -574,7 +580,7 @@ __device__ __forceinline__ void chart_tile(const UfArgs& a, uint32_t tile, const
     }
     if (w < nwords && t < a.T) tri_chart[t] = chart[k];
   }
-  put_visible<NT>(words, __ldcg(visstart + tile), chart, vis, tile);
+  put_visible<NT>(words, start, chart, vis, tile);
 }
 
 // Every counting block (a block each; invisible triangles get -1), or, when the
@@ -586,14 +592,16 @@ __device__ __forceinline__ void tri_chart_body(const UfArgs& a, const uint32_t* 
                                                uint32_t* box_full, uint32_t max_charts, const uint32_t* visstart,
                                                uint2* vis, uint32_t bid, uint32_t nblk) {
   __shared__ int32_t s_status;
+  uint32_t next = LIST ? list_entry(a, bid) : 0u;
+  const uint32_t n = LIST ? __ldcg(&a.ctr->n_vtiles) : (a.T + kPerBlock - 1) / kPerBlock;
   if (threadIdx.x == 0) s_status = __ldcg(&a.ctr->status);
   __syncthreads();
   if (s_status != 0) return;
-  const uint32_t n = LIST ? __ldcg(&a.ctr->n_vtiles) : (a.T + kPerBlock - 1) / kPerBlock;
   for (uint32_t i = bid; i < n; i += nblk) {
+    const uint32_t tile = LIST ? next : i;
+    if (LIST) next = list_entry(a, i + nblk);
     __syncthreads();  // the shared memory of the previous tile is free
-    chart_tile<NT>(a, LIST ? __ldcg(a.tile_list + i) : i, blockcnt, wordroots, tri_chart, roots, box_enc, box_full,
-                   max_charts, visstart, vis);
+    chart_tile<NT>(a, tile, blockcnt, wordroots, tri_chart, roots, box_enc, box_full, max_charts, visstart, vis);
   }
 }
 

@@ -272,13 +272,12 @@ struct FootArgs {
   uint8_t* rot;
 };
 
-__device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t c) {
+__device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t c, uint32_t full, uint4 e) {
   float x0, y0, x1, y1;
-  if (__ldcg(f.box_full + c)) {
+  if (full) {
     x0 = y0 = -1.0f;
     x1 = y1 = 1.0f;
   } else {
-    const uint4 e = __ldcg(reinterpret_cast<const uint4*>(f.box_enc) + c);
     x0 = unordered(e.x);
     y0 = unordered(e.y);
     x1 = unordered(e.z);
@@ -294,6 +293,10 @@ __device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t 
   f.fa[c] = r ? fh : fw;
   f.fb[c] = r ? fw : fh;
   return r ? fw : fh;
+}
+
+__device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t c) {
+  return chart_footprint(f, c, __ldcg(f.box_full + c), __ldcg(reinterpret_cast<const uint4*>(f.box_enc) + c));
 }
 
 __device__ __forceinline__ void set_status(DevCounters* c, int32_t s) {
@@ -378,12 +381,13 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
 fa_status launch_chartify(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* vt, uint32_t mode,
                           int32_t* tri_chart, int32_t* vert_chart, const fa_charts* ch,
                           cudaStream_t s, bool tile_list = false, bool tri_chart_cleared = false);
-// launch_parameterize and launch_uv read the context's visible-triangle list (built
-// by chartify, or by launch_vis_list).
+// launch_parameterize and launch_uv read the context's visible-triangle list (built by
+// chartify), or, when not listed (the standalone calls), walk tri_chart.
 fa_status launch_parameterize(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W,
                               uint32_t H, float ratio, const int32_t* tri_chart,
                               const fa_charts* ch, bool reset_boxes, uint32_t flags, uint32_t* partial,
-                              cudaStream_t s, const float* Mdev = nullptr, bool footprint = true);
+                              cudaStream_t s, const float* Mdev = nullptr, bool footprint = true,
+                              bool listed = true);
 // Footprint inputs / outputs of the charts of ch (fused into the first order kernel
 // on the frame path).
 FootArgs foot_args(fa_ctx* ctx, uint32_t W, uint32_t H, float ratio, const fa_charts* ch);
@@ -395,10 +399,8 @@ fa_status launch_uv(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W,
                     float ratio, const int32_t* tri_chart, const fa_charts* ch,
                     const fa_placement* place, const fa_pack_result* res, uint32_t atlas_log2,
                     uint32_t n_scales, float* uv, float* affine, cudaStream_t s,
-                    const float* Mdev = nullptr, bool from_candidates = false);
+                    const float* Mdev = nullptr, bool from_candidates = false, bool listed = true);
 fa_status build_adjacency(fa_ctx* ctx, fa_mesh* mesh, cudaStream_t s);
-// The visible-triangle list from a caller's tri_chart (standalone box / UV calls).
-fa_status launch_vis_list(fa_ctx* ctx, const fa_mesh* mesh, const int32_t* tri_chart, cudaStream_t s);
 // One whole frame on ctx: host-side checks, then the launch sequence.
 fa_status check_frame(const fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params* p, const float* d_view_proj,
                       const fa_frame_out* o);

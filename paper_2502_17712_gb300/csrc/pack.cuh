@@ -88,15 +88,23 @@ __device__ __forceinline__ T block_max(T v, T* warp_vals) {
 template <bool FOOT>
 __device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint32_t* __restrict__ fb,
                                                 const FootArgs& foot, uint32_t bid, uint32_t* hist) {
-  if (__ldcg(&p.ctr->status) != 0) return;
+  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const uint32_t i = bid * kOrderTile + tid;
+  // the accumulators of chart i (of an earlier frame, past the count), the count and the
+  // status word at once; a caller's fb only has room for the count
+  uint32_t full = 0;
+  uint4 enc = make_uint4(0u, 0u, 0u, 0u);
+  if (FOOT && i < p.max_boxes) {
+    full = __ldcg(foot.box_full + i);
+    enc = __ldcg(reinterpret_cast<const uint4*>(foot.box_enc) + i);
+  }
   const uint32_t C = __ldcg(p.count);
+  if (__ldcg(&p.ctr->status) != 0) return;
   if (C > p.max_boxes) return;
   const uint32_t ntiles = (C + kOrderTile - 1) / kOrderTile;
   if (bid >= ntiles) return;
-  const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const uint32_t i = bid * kOrderTile + tid;
   uint32_t fbi = 0;
-  if (i < C) fbi = FOOT ? chart_footprint(foot, i) : __ldg(fb + i);
+  if (i < C) fbi = FOOT ? chart_footprint(foot, i, full, enc) : __ldg(fb + i);
   const uint32_t bin = i < C ? height_bin(fbi) : kMaxH;  // kMaxH: no box
   for (uint32_t b = tid; b < kMaxH; b += kOrderTile) hist[b] = 0;
   // stable rank inside the tile: the warps take their turn in index order; inside a
@@ -132,14 +140,6 @@ __device__ __forceinline__ void order_scatter_body(const PackScratch& p, const u
                                                    const uint32_t* __restrict__ fb, uint32_t* order, uint32_t bid,
                                                    uint32_t* binstart) {
   __shared__ uint32_t wt[32];
-  if (__ldcg(&p.ctr->status) != 0) return;
-  const uint32_t C = __ldcg(p.count);
-  if (C > p.max_boxes) return;
-  if (bid == 0) {  // also with no boxes: the push reads the overflows
-    for (uint32_t i = threadIdx.x; i < kMaxScales * p.max_chunks; i += blockDim.x) p.scan_state[i] = 0ull;
-    if (threadIdx.x < kMaxScales) p.m[threadIdx.x] = 0u;
-  }
-  if (bid * kOrderTile >= C) return;
   constexpr uint32_t kPer = kMaxH / kOrderTile;
   const uint4* t4 = reinterpret_cast<const uint4*>(p.ord_total) + threadIdx.x * (kPer / 4);
   uint32_t v[kPer];
@@ -150,6 +150,21 @@ __device__ __forceinline__ void order_scatter_body(const PackScratch& p, const u
     v[4 * j + 1] = q.y;
     v[4 * j + 2] = q.z;
     v[4 * j + 3] = q.w;
+  }
+  const uint32_t C = __ldcg(p.count);
+  if (__ldcg(&p.ctr->status) != 0) return;
+  if (C > p.max_boxes) return;
+  if (bid == 0) {  // also with no boxes: the push reads the overflows
+    for (uint32_t i = threadIdx.x; i < kMaxScales * p.max_chunks; i += blockDim.x) p.scan_state[i] = 0ull;
+    if (threadIdx.x < kMaxScales) p.m[threadIdx.x] = 0u;
+  }
+  if (bid * kOrderTile >= C) return;
+  const uint32_t i = bid * kOrderTile + threadIdx.x;
+  uint32_t fai = 0, fbi = 0, rank = 0;  // (on their way during the scan)
+  if (i < C) {
+    fai = __ldcg(fa + i);
+    fbi = __ldcg(fb + i);
+    rank = __ldcg(p.ord_rank + i);
   }
   uint32_t sum = 0;
 #pragma unroll
@@ -162,10 +177,9 @@ __device__ __forceinline__ void order_scatter_body(const PackScratch& p, const u
     run += v[j];
   }
   __syncthreads();
-  const uint32_t i = bid * kOrderTile + threadIdx.x;
   if (i >= C) return;
-  const uint32_t bin = height_bin(__ldcg(fb + i));
-  uint32_t pos = binstart[bin] + p.ord_rank[i];
+  const uint32_t bin = height_bin(fbi);
+  uint32_t pos = binstart[bin] + rank;
   // the bin's boxes in earlier tiles: sixteen independent loads per round
   for (uint32_t t = 0; t < bid; t += 16) {
     const uint32_t* c = p.ord_counts + (size_t)t * kMaxH + bin;
@@ -177,7 +191,7 @@ __device__ __forceinline__ void order_scatter_body(const PackScratch& p, const u
   }
   if (pos < C) {
     order[pos] = i;
-    p.fs[pos] = make_uint2(__ldcg(fa + i), __ldcg(fb + i));
+    p.fs[pos] = make_uint2(fai, fbi);
   }
   p.ord_rank[i] = pos;  // from here on: the box's position in the order
 }
@@ -508,10 +522,10 @@ __device__ __forceinline__ void pack_scan_body(const PackScratch& p, const PackA
   __shared__ int32_t s_status;
   // one read of the status word for the whole CTA (another CTA's time-out can set
   // it meanwhile, and every thread must take the same branch before the barriers)
+  const uint32_t C = __ldcg(p.count);
   if (threadIdx.x == 0) s_status = __ldcg(&p.ctr->status);
   __syncthreads();
   if (s_status != 0) return;
-  const uint32_t C = __ldcg(p.count);
   if (C > p.max_boxes || C == 0) return;
   if (PAIRS && (unsigned long long)((C + kChunk - 1) / kChunk) * n_scales > nblk)
     pack_scan_items<NT, 2>(p, a, n_scales, C, bid, nblk);
@@ -598,11 +612,12 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
   // no work, but every CTA still publishes and counts itself, so that the last one
   // selects and resets the counter.  One read for the whole CTA: every thread must
   // take the same branch before the barriers below.
+  const uint32_t om = 1u << a.atlas_log2;
+  const uint32_t C = __ldcg(p.count), over = __ldcg(p.m + kidx);
   if (tid == 0) s_st0 = __ldcg(&p.ctr->status);
+  for (uint32_t x = tid; x < om; x += NT) F[x] = 0;  // (while the loads are on their way)
   __syncthreads();
   const int32_t st0 = s_st0;
-  const uint32_t C = __ldcg(p.count);
-  const uint32_t om = 1u << a.atlas_log2;
   int32_t status = FA_OK;
   uint32_t Om = om, H = 0, ok = 0;
   if (st0 != 0) {
@@ -610,7 +625,7 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
   } else if (C > p.max_boxes) {
     status = FA_E_CAPACITY;
   } else {
-    Om = om + __ldcg(p.m + kidx);
+    Om = om + over;
     if (Om > a.front_cap) {
       status = FA_E_CAPACITY;
     } else {
@@ -627,7 +642,7 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
         bulk_g2s(dst, rec + (size_t)c * kChunk, rbytes, &s_bar[c & 1u]);
         bulk_g2s(dst + kChunk * 8u, sgg + (size_t)c * kSegStride, kSegStride * 2u, &s_bar[c & 1u]);
       };
-      for (uint32_t x = tid; x < Om; x += NT) F[x] = 0;
+      for (uint32_t x = om + tid; x < Om; x += NT) F[x] = 0;
       if (tid == 0) {
         mbar_init(&s_bar[0], 1);
         mbar_init(&s_bar[1], 1);

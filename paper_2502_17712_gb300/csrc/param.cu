@@ -56,14 +56,14 @@ FootArgs foot_args(fa_ctx* ctx, uint32_t W, uint32_t H, float ratio, const fa_ch
 fa_status launch_parameterize(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W, uint32_t H,
                               float ratio, const int32_t* tri_chart, const fa_charts* ch, bool reset_boxes,
                               uint32_t flags, uint32_t* partial, cudaStream_t s, const float* Mdev,
-                              bool footprint) {
+                              bool footprint, bool listed) {
   if (partial) FA_CUDA_TRY(cudaMemsetAsync(partial, 0, (size_t)((mesh->T + 31) / 32) * 4, s));
   if (reset_boxes) {
     mark(ctx, "k_box_reset", s);
     launch_k(k_box_reset, grid_for(ctx->cfg.max_charts, 256, 152 * 4), 256, 0, s, ch->count, ctx->cfg.max_charts,
                                                                             ctx->box_enc, ctx->box_full);
   }
-  const BoxArgs a = pm::make_box_args(ctx, mesh, M, tri_chart, flags, partial, Mdev);
+  const BoxArgs a = pm::make_box_args(ctx, mesh, M, tri_chart, flags, partial, Mdev, listed);
   mark(ctx, "k_bbox", s);
   if (Mdev)
     launch_k(k_bbox<true>, grid_for(mesh->T, 256, 152 * 8), 256, 0, s, a);
@@ -82,9 +82,9 @@ fa_status launch_uv(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W,
                     const int32_t* tri_chart, const fa_charts* ch,
                     const fa_placement* place, const fa_pack_result* res, uint32_t atlas_log2,
                     uint32_t n_scales, float* uv, float* affine, cudaStream_t s, const float* Mdev,
-                    bool from_candidates) {
+                    bool from_candidates, bool listed) {
   const UvArgs a = pm::make_uv_args(ctx, mesh, M, W, H, ratio, tri_chart, ch, place, res, atlas_log2, n_scales, uv,
-                                    affine, Mdev, from_candidates);
+                                    affine, Mdev, from_candidates, listed);
   mark(ctx, "k_uv", s);
   if (Mdev)
     launch_k(k_uv<true>, grid_for(mesh->T, 256, 152 * 8), 256, 0, s, a);

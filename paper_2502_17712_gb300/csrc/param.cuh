@@ -65,7 +65,7 @@ struct BoxArgs {
   const float* Mdev;  // when set, the matrix is read here on the device instead of M
   const float* pos;
   const uint32_t* idx;
-  const uint2* vis;  // (triangle, chart) of the visible triangles
+  const uint2* vis;  // (triangle, chart) of the visible triangles, or null: tri_chart is walked
   const int32_t* tri_chart;
   uint32_t T;
   uint32_t* box_enc;
@@ -73,6 +73,14 @@ struct BoxArgs {
   uint32_t max_charts;
   DevCounters* ctr;
 };
+
+// Entry i of the visible-triangle list; without a list (a caller's tri_chart), triangle
+// i and its chart, -1 where it is not visible.
+template <class Args>
+__device__ __forceinline__ uint2 vis_entry(const Args& a, uint32_t i) {
+  if (i >= a.T) return make_uint2(0xFFFFFFFFu, 0xFFFFFFFFu);
+  return a.vis ? __ldcg(a.vis + i) : make_uint2(i, (uint32_t)__ldg(a.tri_chart + i));
+}
 
 // Signed distance to frustum plane pl (inside iff >= 0): 0 left x >= -w, 1 right
 // x <= w, 2 bottom y >= -w, 3 top y <= w, 4 far z <= w.
@@ -138,19 +146,24 @@ __device__ __forceinline__ void box_frustum(Box& b, const CV (&v)[3]) {
 template <bool DEV_M>
 __device__ __forceinline__ void bbox_body(const BoxArgs& a, uint32_t bid, uint32_t nblk) {
   const Mat4 M = DEV_M ? load_mat(a.Mdev) : a.M;
-  if (__ldcg(&a.ctr->status) != 0) return;
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t n = __ldcg(&a.ctr->n_vis);
   const uint32_t stride = nblk * blockDim.x;
-  for (uint32_t base = bid * blockDim.x + (threadIdx.x & ~31u); base < n; base += stride) {
+  const uint32_t base0 = bid * blockDim.x + (threadIdx.x & ~31u);
+  // the first list entry (left from an earlier frame, if the list is shorter), the
+  // list's length and the status word at once
+  uint2 next = vis_entry(a, base0 + lane);
+  const uint32_t n = a.vis ? __ldcg(&a.ctr->n_vis) : a.T;
+  if (__ldcg(&a.ctr->status) != 0) return;
+  for (uint32_t base = base0; base < n; base += stride) {
     const uint32_t i = base + lane;
+    const uint2 e = next;
+    next = vis_entry(a, i + stride);
     uint32_t t = 0;
     int32_t c = -1;
     Box b{__int_as_float(0x7f800000), __int_as_float(0x7f800000), __int_as_float(0xff800000),
           __int_as_float(0xff800000), false};
     bool pv = false;  // partially visible (Sec. 6): a vertex with max(|x|, |y|) >= w
     if (i < n) {
-      const uint2 e = __ldcg(a.vis + i);
       t = e.x;
       c = (int32_t)e.y;
       if ((uint32_t)c >= a.max_charts || t >= a.T) c = -1;  // not a chart of this context: ignored
@@ -254,7 +267,7 @@ struct UvArgs {
   const float* Mdev;  // when set, the matrix is read here on the device instead of M
   const float* pos;
   const uint32_t* idx;
-  const uint2* vis;  // (triangle, chart) of the visible triangles
+  const uint2* vis;  // (triangle, chart) of the visible triangles, or null: tri_chart is walked
   const int32_t* tri_chart;
   uint32_t T;
   float hx, hy;
@@ -291,9 +304,13 @@ __device__ __forceinline__ fa_placement placement_of(const UvArgs& a, uint32_t c
 template <bool DEV_M>
 __device__ __forceinline__ void uv_body(const UvArgs& a, uint32_t bid, uint32_t nblk) {
   const Mat4 M = DEV_M ? load_mat(a.Mdev) : a.M;
-  if (__ldcg(&a.ctr->status) != 0 || __ldcg(&a.res->status) != FA_OK) return;
-  const uint32_t k = __ldcg(&a.res->k);
-  const float om = (float)(1u << a.atlas_log2), Om = (float)__ldcg(&a.res->omega);
+  // every word that the first loads below depend on, at once
+  const int32_t st = __ldcg(&a.ctr->status), rst = __ldcg(&a.res->status);
+  const uint32_t k = __ldcg(&a.res->k), omega = __ldcg(&a.res->omega);
+  const uint32_t n = a.vis ? __ldcg(&a.ctr->n_vis) : a.T;
+  const uint32_t C = min(__ldcg(a.count), a.max_charts);
+  if (st != 0 || rst != FA_OK) return;
+  const float om = (float)(1u << a.atlas_log2), Om = (float)omega;
   const DF alpha = df_div(om, Om);
   DF g = quick_two_sum(__fmul_rn(a.ratio, (float)k), __fmaf_rn(a.ratio, (float)k, -__fmul_rn(a.ratio, (float)k)));
   const float inv_n = 1.0f / (float)a.n_scales;  // power of two: exact
@@ -310,7 +327,6 @@ __device__ __forceinline__ void uv_body(const UvArgs& a, uint32_t bid, uint32_t 
   const uint32_t tri_blocks = nblk - chart_blocks;
   // per chart: the placement (frame path) and the affine (uv = A . ndc + b)
   if (per_chart && (chart_blocks == 0u || bid >= tri_blocks)) {
-    const uint32_t C = min(__ldcg(a.count), a.max_charts);
     const uint32_t c0 = (chart_blocks ? bid - tri_blocks : bid) * blockDim.x + threadIdx.x;
     const uint32_t cstride = (chart_blocks ? chart_blocks : nblk) * blockDim.x;
     for (uint32_t c = c0; c < C; c += cstride) {
@@ -340,23 +356,27 @@ __device__ __forceinline__ void uv_body(const UvArgs& a, uint32_t bid, uint32_t 
     }
   }
   if (!a.uv || bid >= tri_blocks) return;
-  const uint32_t n = __ldcg(&a.ctr->n_vis);
-  const uint32_t C = min(__ldcg(a.count), a.max_charts);
-  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < n; i += tri_blocks * blockDim.x) {
-    const uint2 e = __ldcg(a.vis + i);
+  const uint32_t stride = tri_blocks * blockDim.x;
+  uint2 next = vis_entry(a, bid * blockDim.x + threadIdx.x);
+  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const uint2 e = next;
+    next = vis_entry(a, i + stride);
     const uint32_t t = e.x;
     const int32_t c = (int32_t)e.y;
     if (c < 0 || (uint32_t)c >= C || t >= a.T) continue;
+    // the corner indices beside the chart's words, then the corners beside its placement
+    const uint32_t* f = a.idx + 3 * (size_t)t;
+    const uint32_t f0 = __ldg(f), f1 = __ldg(f + 1), f2 = __ldg(f + 2);
     const float4 bb = reinterpret_cast<const float4*>(a.bbox)[c];
-    const fa_placement pl = placement_of(a, c, kb);
     const bool r = __ldcg(a.rot + c) != 0;
+    const fa_placement pl = placement_of(a, c, kb);
+    const float4 cl[3] = {load_clip(M, a.pos, f0), load_clip(M, a.pos, f1), load_clip(M, a.pos, f2)};
     const DF X = two_sum((float)pl.x, gut), Y = two_sum((float)pl.y, gut);
     const DF wpx = df_mul_f(two_sum(bb.z, -bb.x), a.hx);
-    const uint32_t* f = a.idx + 3 * (size_t)t;
     float2* o = reinterpret_cast<float2*>(a.uv + 6 * (size_t)t);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const float4 cc = load_clip(M, a.pos, __ldg(f + j));
+      const float4 cc = cl[j];
       if (!(cc.w > 0.0f)) {
         o[j] = make_float2(__int_as_float(0x7fffffff), __int_as_float(0x7fffffff));
         continue;
@@ -381,7 +401,7 @@ __device__ __forceinline__ void uv_body(const UvArgs& a, uint32_t bid, uint32_t 
 // The box-pass arguments on ctx (host side); the pass walks the context's
 // visible-triangle list.
 inline BoxArgs make_box_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, const int32_t* tri_chart,
-                             uint32_t flags, uint32_t* partial, const float* Mdev) {
+                             uint32_t flags, uint32_t* partial, const float* Mdev, bool listed = true) {
   BoxArgs a;
   a.M = M;
   a.Mdev = Mdev;
@@ -389,7 +409,7 @@ inline BoxArgs make_box_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, co
   a.partial = partial;
   a.pos = mesh->pos;
   a.idx = mesh->idx;
-  a.vis = ctx->vis;
+  a.vis = listed ? ctx->vis : nullptr;
   a.tri_chart = tri_chart;
   a.T = mesh->T;
   a.box_enc = ctx->box_enc;
@@ -404,13 +424,13 @@ inline BoxArgs make_box_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, co
 inline UvArgs make_uv_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W, uint32_t H, float ratio,
                            const int32_t* tri_chart, const fa_charts* ch, const fa_placement* place,
                            const fa_pack_result* res, uint32_t atlas_log2, uint32_t n_scales, float* uv,
-                           float* affine, const float* Mdev, bool from_candidates) {
+                           float* affine, const float* Mdev, bool from_candidates, bool listed = true) {
   UvArgs a;
   a.M = M;
   a.Mdev = Mdev;
   a.pos = mesh->pos;
   a.idx = mesh->idx;
-  a.vis = ctx->vis;
+  a.vis = listed ? ctx->vis : nullptr;
   a.tri_chart = tri_chart;
   a.T = mesh->T;
   a.hx = 0.5f * (float)W;

@@ -1416,6 +1416,11 @@ template <bool DEV_M, int NT>
 __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
   uint32_t* pre = region_pre();
   const uint32_t lane = threadIdx.x & 31;
+  // (the clipped triangles' counts with the survivors': mostly there are none)
+  uint32_t clipped = 0;
+#pragma unroll
+  for (uint32_t j = 0; j < (kMaxFrontBlocks + NT - 1) / NT; ++j)
+    if (threadIdx.x + j * NT < A.front_blocks) clipped |= __ldcg(A.clip_count + threadIdx.x + j * NT);
   const uint32_t n = surv_prefix<NT>(A, pre);
   const uint32_t stride = nblk * blockDim.x;
   const bool grouped = (uint64_t)n * kRasterGroup <= (uint64_t)stride;  // few survivors: see exact_body
@@ -1499,7 +1504,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
     }
   }
   // then the (rare) triangles that need clipping, from the front blocks' regions
-  __syncthreads();  // pre is reused
+  if (!__syncthreads_or(clipped != 0u)) return;  // (and pre is reused)
   const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
   for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
     const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
@@ -1515,6 +1520,7 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
   __shared__ uint32_t pre[kMidLists + 1];
   const uint32_t lane = threadIdx.x & 31;
   __syncthreads();  // pre of an earlier item of the same block is free
+  const unsigned long long st = __ldcg(&A.ctr->big);
   if (threadIdx.x < 32) {
     uint32_t c = 0;
     if (lane < A.mid_lists) c = min(__ldcg(&A.ctr->n_mid[lane][0]), mid_base(A, lane + 1u) - mid_base(A, lane));
@@ -1528,7 +1534,6 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
     if (lane == 0) pre[0] = 0u;
   }
   const uint32_t warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = (nblk * blockDim.x) >> 5;
-  const unsigned long long st = __ldcg(&A.ctr->big);
   const uint32_t n_ent = (uint32_t)min((unsigned long long)A.queue_cap, st >> 40);
   const uint32_t n_tiles = n_ent ? (uint32_t)min((unsigned long long)A.tile_cap, st & ((1ull << 40) - 1)) : 0u;
   for (uint32_t g = warp; g < n_tiles; g += nwarps) {
