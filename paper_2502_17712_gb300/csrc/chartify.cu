@@ -31,11 +31,6 @@ void launch_local(uint32_t nt, uint32_t ntiles, cudaStream_t s, const UfArgs& a)
     launch_k(k_uf_local<LIST, 1024>, grid(2), 1024, 0, s, a);
 }
 
-__global__ void k_uf_init_v(int32_t* label, uint32_t T, uint32_t V) {
-  pdl_wait();
-  cf::init_v_body(label, T, V, blockIdx.x, gridDim.x);
-}
-
 template <bool LIST>
 __global__ void __launch_bounds__(128) k_uf_hook(UfArgs a) {
   pdl_wait();
@@ -87,13 +82,10 @@ __global__ void k_vert_chart(UfArgs a, const uint32_t* blockcnt, const uint2* wo
 fa_status launch_chartify(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* vt, uint32_t mode,
                           int32_t* tri_chart, int32_t* vert_chart, const fa_charts* ch, cudaStream_t s,
                           bool tile_list, bool tri_chart_cleared) {
-  const UfArgs a = cf::make_uf_args(ctx, mesh, vt);
+  UfArgs a = cf::make_uf_args(ctx, mesh, vt);
   const int vm = mode == FA_CHARTS_VERTEX;
+  a.init_v = vm ? 1u : 0u;
   const unsigned gw = grid_for((uint64_t)((mesh->T + 31) / 32) * 32, kBlock, 152 * 16);
-  if (vm) {
-    mark(ctx, "k_uf_init_v", s);
-    launch_k(k_uf_init_v, grid_for(mesh->V, 256, 152 * 8), 256, 0, s, ctx->label, mesh->T, mesh->V);
-  }
   const uint32_t ntiles = (mesh->T + kTile - 1) / kTile;
   mark(ctx, "k_uf_local", s);
   if (tile_list)

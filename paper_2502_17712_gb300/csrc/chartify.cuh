@@ -94,6 +94,7 @@ struct UfArgs {
   const uint32_t* tile_list;  // tiles with a visible triangle (count in ctr->n_vtiles)
   DevCounters* ctr;
   uint32_t loop_cap;  // CAS retries of one hooking step before FA_E_TIMEOUT
+  uint32_t init_v;    // the local pass also sets the vertex nodes' labels (vertex mode)
 };
 
 // Union of the edges inside one tile of kTile consecutive triangles, in shared
@@ -209,6 +210,11 @@ __device__ __forceinline__ void local_tile(const UfArgs& a, uint32_t tile) {
   if (threadIdx.x == 0) a.xcnt[tile] = s_xc;  // all appends precede the last barrier
 }
 
+__device__ __forceinline__ void init_v_body(int32_t* label, uint32_t T, uint32_t V, uint32_t bid, uint32_t nblk) {
+  for (uint32_t v = bid * blockDim.x + threadIdx.x; v < V; v += nblk * blockDim.x)
+    label[T + v] = (int32_t)(T + v);
+}
+
 // Entry i of the tile list, or anything past its room: read before the list's length is
 // known, so that the two loads do not wait for one another (a frame's kernels are chains
 // of such loads, about 0.4 us each).
@@ -220,6 +226,7 @@ __device__ __forceinline__ uint32_t list_entry(const UfArgs& a, uint32_t i) {
 // persistent grid over the list).
 template <bool LIST, int NT>
 __device__ __forceinline__ void local_body(const UfArgs& a, uint32_t bid, uint32_t nblk) {
+  if (a.init_v) init_v_body(a.label, a.T, a.V, bid, nblk);
   if (!LIST) {
     const uint32_t ntiles = (a.T + kTile - 1) / kTile;
     for (uint32_t t = bid; t < ntiles; t += nblk) {
@@ -241,11 +248,6 @@ __device__ __forceinline__ void local_body(const UfArgs& a, uint32_t bid, uint32
     __syncthreads();
     i = s_i;
   }
-}
-
-__device__ __forceinline__ void init_v_body(int32_t* label, uint32_t T, uint32_t V, uint32_t bid, uint32_t nblk) {
-  for (uint32_t v = bid * blockDim.x + threadIdx.x; v < V; v += nblk * blockDim.x)
-    label[T + v] = (int32_t)(T + v);
 }
 
 // Hooking (Alg. 1, second loop), edge mode: the edges that leave a tile, each once
@@ -283,7 +285,11 @@ __device__ __forceinline__ void hook_body(const UfArgs& a, uint32_t bid, uint32_
   }
 }
 
-// Vertex mode: every visible triangle joins its three vertex nodes T + v.
+// Vertex mode: every visible triangle joins its three vertex nodes T + v.  A vertex node
+// takes the smallest tile-local root of its triangles (atomicMin); a triangle that finds
+// another root there joins it.  Every root that comes to a vertex after the first is so
+// joined with one that came before, and most find their own: one atomic a corner instead
+// of two walks and a CAS (322,118 visible triangles of 128 patches: 42.6 -> 20.3 us).
 __device__ __forceinline__ void hook_v_body(const UfArgs& a, uint32_t bid, uint32_t nblk) {
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t nwords = (a.T + 31) >> 5;
@@ -292,11 +298,16 @@ __device__ __forceinline__ void hook_v_body(const UfArgs& a, uint32_t bid, uint3
     if (word == 0) continue;
     const uint32_t t = (w << 5) + lane;
     if (!((word >> lane) & 1u)) continue;
+    const int32_t r = __ldcg(a.label + t);
+    uint32_t v[3];
+    int32_t old[3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      uint32_t v = __ldg(a.idx + 3 * (size_t)t + j);
-      unite(a.label, (int32_t)t, (int32_t)(a.T + v), a.ctr, a.loop_cap);
-    }
+    for (int j = 0; j < 3; ++j) v[j] = __ldg(a.idx + 3 * (size_t)t + j);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) old[j] = atomicMin(a.label + a.T + v[j], r);
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (old[j] < (int32_t)a.T && old[j] != r) unite(a.label, r, old[j], a.ctr, a.loop_cap);
   }
 }
 
@@ -632,6 +643,7 @@ inline UfArgs make_uf_args(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* vt)
   a.tile_list = ctx->tile_list;
   a.ctr = ctx->ctr;
   a.loop_cap = ctx->loop_cap;
+  a.init_v = 0u;
   return a;
 }
 
