@@ -261,7 +261,7 @@ __device__ __forceinline__ float unordered(uint32_t k) {
 
 // Footprint of chart c from its box accumulators (Sec. 5.2, Sec. 4.1): the box
 // (full: [-1, 1]^2), its viewport size scaled by 256 * ratio and rounded up to 1/256
-// texel, rotated to stand tall.  Written to bbox / fa / fb / rot; returns fb.
+// texel, rotated to stand tall.  Written to bbox / fa / fb / rot; returns (fa, fb).
 struct FootArgs {
   const uint32_t* box_enc;
   const uint32_t* box_full;
@@ -272,7 +272,7 @@ struct FootArgs {
   uint8_t* rot;
 };
 
-__device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t c, uint32_t full, uint4 e) {
+__device__ __forceinline__ uint2 chart_footprint(const FootArgs& f, uint32_t c, uint32_t full, uint4 e) {
   float x0, y0, x1, y1;
   if (full) {
     x0 = y0 = -1.0f;
@@ -290,12 +290,13 @@ __device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t 
   const uint32_t fh = __float2uint_rz(ceilf(__fmul_rn(f.s256, hpx)));
   const bool r = fw > fh;
   f.rot[c] = r ? 1 : 0;
-  f.fa[c] = r ? fh : fw;
-  f.fb[c] = r ? fw : fh;
-  return r ? fw : fh;
+  const uint2 s = r ? make_uint2(fh, fw) : make_uint2(fw, fh);
+  f.fa[c] = s.x;
+  f.fb[c] = s.y;
+  return s;
 }
 
-__device__ __forceinline__ uint32_t chart_footprint(const FootArgs& f, uint32_t c) {
+__device__ __forceinline__ uint2 chart_footprint(const FootArgs& f, uint32_t c) {
   return chart_footprint(f, c, __ldcg(f.box_full + c), __ldcg(reinterpret_cast<const uint4*>(f.box_enc) + c));
 }
 

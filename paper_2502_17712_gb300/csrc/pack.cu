@@ -9,11 +9,12 @@ namespace {
 using pk::PackArgs;
 
 template <bool FOOT>
-__global__ void __launch_bounds__(kOrderTile) k_order_tile(PackScratch p, const uint32_t* __restrict__ fb,
-                                                           FootArgs foot) {
+__global__ void __launch_bounds__(kOrderTile) k_order_tile(PackScratch p, const uint32_t* __restrict__ fa,
+                                                           const uint32_t* __restrict__ fb, FootArgs foot,
+                                                           uint32_t* order) {
   pdl_wait();
   __shared__ uint32_t hist[kMaxH];
-  pk::order_tile_body<FOOT>(p, fb, foot, blockIdx.x, hist);
+  pk::order_tile_body<FOOT>(p, fa, fb, foot, order, blockIdx.x, hist);
 }
 
 __global__ void __launch_bounds__(kOrderTile) k_order_scatter(PackScratch p, const uint32_t* __restrict__ fa,
@@ -49,9 +50,9 @@ fa_status launch_pack_kernels(fa_ctx* ctx, const PackScratch& p, const uint32_t*
   uint32_t* ord = order ? order : p.order;
   if (ctx) mark(ctx, "k_order_tile", s);
   if (foot)
-    launch_k(k_order_tile<true>, p.max_tiles, kOrderTile, 0, s, p, fb, *foot);
+    launch_k(k_order_tile<true>, p.max_tiles, kOrderTile, 0, s, p, fa_, fb, *foot, ord);
   else
-    launch_k(k_order_tile<false>, p.max_tiles, kOrderTile, 0, s, p, fb, FootArgs{});
+    launch_k(k_order_tile<false>, p.max_tiles, kOrderTile, 0, s, p, fa_, fb, FootArgs{}, ord);
   if (ctx) mark(ctx, "k_order_scatter", s);
   launch_k(k_order_scatter, p.max_tiles, kOrderTile, 0, s, p, fa_, fb, ord);
   const PackArgs a = pk::make_pack_args(ctx, ord, atlas_log2, n_scales, select_mode, min_box, gutter, lowres_log2,

@@ -85,9 +85,13 @@ __device__ __forceinline__ T block_max(T v, T* warp_vals) {
 // FOOT: the charts' footprints are computed here from their box accumulators
 // (written out, and their heights used as the keys) instead of read from fb.
 // hist: kMaxH words of shared memory (boxes of each height bin seen so far in the tile).
+// Boxes of one tile (C <= kOrderTile) are put in order here, from the tile's own bins;
+// k_order_scatter then has nothing to do (7,938-triangle frame 67 -> 65 us).
 template <bool FOOT>
-__device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint32_t* __restrict__ fb,
-                                                const FootArgs& foot, uint32_t bid, uint32_t* hist) {
+__device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint32_t* __restrict__ fa,
+                                                const uint32_t* __restrict__ fb, const FootArgs& foot,
+                                                uint32_t* order, uint32_t bid, uint32_t* hist) {
+  __shared__ uint32_t wt[32];
   const uint32_t tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const uint32_t i = bid * kOrderTile + tid;
   // the accumulators of chart i (of an earlier frame, past the count), the count and the
@@ -103,9 +107,12 @@ __device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint
   if (C > p.max_boxes) return;
   const uint32_t ntiles = (C + kOrderTile - 1) / kOrderTile;
   if (bid >= ntiles) return;
-  uint32_t fbi = 0;
-  if (i < C) fbi = FOOT ? chart_footprint(foot, i, full, enc) : __ldg(fb + i);
-  const uint32_t bin = i < C ? height_bin(fbi) : kMaxH;  // kMaxH: no box
+  uint2 f = make_uint2(0u, 0u);  // (fa only for one tile)
+  if (i < C) {
+    if (FOOT) f = chart_footprint(foot, i, full, enc);
+    else f = make_uint2(ntiles == 1u ? __ldg(fa + i) : 0u, __ldg(fb + i));
+  }
+  const uint32_t bin = i < C ? height_bin(f.y) : kMaxH;  // kMaxH: no box
   for (uint32_t b = tid; b < kMaxH; b += kOrderTile) hist[b] = 0;
   // stable rank inside the tile: the warps take their turn in index order; inside a
   // warp, the lanes with the same bin are ranked by lane
@@ -113,7 +120,8 @@ __device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint
   const uint32_t before = __popc(peers & ((1u << lane) - 1u));
   const bool leader = before == 0u;
   uint32_t r = 0;
-  for (uint32_t w = 0; w < (uint32_t)(kOrderTile / 32); ++w) {
+  const uint32_t turns = (min(C - bid * kOrderTile, (uint32_t)kOrderTile) + 31u) / 32u;
+  for (uint32_t w = 0; w < turns; ++w) {
     __syncthreads();
     if (wid == w && bin < kMaxH) {
       r = hist[bin] + before;
@@ -122,6 +130,30 @@ __device__ __forceinline__ void order_tile_body(const PackScratch& p, const uint
     }
   }
   __syncthreads();
+  if (ntiles == 1u) {
+    // the bins' starts in place (kPer consecutive bins a thread), then the boxes
+    constexpr uint32_t kPer = kMaxH / kOrderTile;
+    uint32_t v[kPer], sum = 0, tot;
+#pragma unroll
+    for (uint32_t j = 0; j < kPer; ++j) {
+      v[j] = hist[tid * kPer + j];
+      sum += v[j];
+    }
+    uint32_t run = block_scan_incl<uint32_t>(sum, wt, &tot) - sum;
+#pragma unroll
+    for (uint32_t j = 0; j < kPer; ++j) {
+      hist[tid * kPer + j] = run;
+      run += v[j];
+    }
+    __syncthreads();
+    if (bin < kMaxH) {
+      const uint32_t pos = hist[bin] + r;
+      order[pos] = i;
+      p.fs[pos] = f;
+      p.ord_rank[i] = pos;
+    }
+    return;
+  }
   if (bin < kMaxH) p.ord_rank[i] = r;
   uint32_t* row = p.ord_counts + (size_t)bid * kMaxH;
   for (uint32_t b = tid; b < kMaxH; b += kOrderTile) {
@@ -158,7 +190,7 @@ __device__ __forceinline__ void order_scatter_body(const PackScratch& p, const u
     for (uint32_t i = threadIdx.x; i < kMaxScales * p.max_chunks; i += blockDim.x) p.scan_state[i] = 0ull;
     if (threadIdx.x < kMaxScales) p.m[threadIdx.x] = 0u;
   }
-  if (bid * kOrderTile >= C) return;
+  if (bid * kOrderTile >= C || C <= kOrderTile) return;  // (one tile: done by k_order_tile)
   const uint32_t i = bid * kOrderTile + threadIdx.x;
   uint32_t fai = 0, fbi = 0, rank = 0;  // (on their way during the scan)
   if (i < C) {
@@ -526,7 +558,7 @@ __device__ __forceinline__ void pack_scan_body(const PackScratch& p, const PackA
   if (threadIdx.x == 0) s_status = __ldcg(&p.ctr->status);
   __syncthreads();
   if (s_status != 0) return;
-  if (C > p.max_boxes || C == 0) return;
+  if (C > p.max_boxes || C <= kChunk) return;  // (one chunk: the push scans it itself)
   if (PAIRS && (unsigned long long)((C + kChunk - 1) / kChunk) * n_scales > nblk)
     pack_scan_items<NT, 2>(p, a, n_scales, C, bid, nblk);
   else
@@ -596,6 +628,66 @@ __device__ __forceinline__ bool better_cand(uint32_t k1, uint32_t o1, uint32_t k
   return l > r || (l == r && k1 > k2);  // larger effective scale, ties to the larger k
 }
 
+// One chunk's boxes for candidate kidx, by the CTA that pushes it: the width scan's work
+// (pack_scan_items) into the first stage, so that no kernel stands between the order and
+// the push (7,938-triangle frame: 67 -> 63 us with the order of one tile).  Returns the
+// largest overflow past omega.  The records also go to global memory, where the
+// placements are read.  (Not inlined: the rows' loop keeps its own registers.)
+template <int NT>
+__device__ __noinline__ uint32_t scan_one_chunk(const uint2* __restrict__ fs, uint2* __restrict__ rec, uint32_t C,
+                                                uint32_t kidx, uint32_t shift, uint32_t min_box, uint32_t gutter,
+                                                uint32_t atlas_log2, uint2* s_rec, uint16_t* s_sg) {
+  __shared__ unsigned long long ws64[32];
+  __shared__ uint32_t ws[32];
+  constexpr int kPer = (int)kChunk / NT;
+  const uint32_t om = 1u << atlas_log2, tid = threadIdx.x, g2 = 2u * gutter;
+  const unsigned long long d = (1ull << shift) - 1ull, k = kidx + 1ull;
+  auto side = [&](uint32_t f) { return max((uint32_t)((k * f + d) >> shift), min_box) + g2; };
+  // consecutive boxes per thread, as few as give every box a thread
+  const uint32_t per = (C + NT - 1u) / NT, j0 = min(tid * per, C), n = min(per, C - j0);
+  uint2 f[kPer];
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) f[e] = (uint32_t)e < n ? __ldcg(fs + j0 + e) : make_uint2(0u, 0u);
+  const uint32_t before = j0 && n ? __ldcg(fs + j0 - 1u).x : 0u;
+  unsigned long long sum = 0, tot64;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
+    f[e].x = (uint32_t)e < n ? side(f[e].x) : 0u;  // from here on: the scaled sides
+    f[e].y = side(f[e].y);
+    sum += f[e].x;
+  }
+  const unsigned long long P0 = block_scan_incl<unsigned long long>(sum, ws64, &tot64) - sum;
+  // a row starts where the box before begins in an earlier row
+  unsigned long long P = P0, prev = j0 ? (P0 - side(before)) >> atlas_log2 : ~0ull;
+  uint32_t starts = 0, cnt = 0, mo = 0, tot;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e) {
+    if ((uint32_t)e >= n) break;
+    const unsigned long long q = P >> atlas_log2;
+    const uint32_t xr = (uint32_t)P & (om - 1u), w = f[e].x;
+    if (q != prev) {
+      starts |= 1u << e;
+      ++cnt;
+    }
+    prev = q;
+    if (xr + w > om) mo = max(mo, xr + w - om);
+    const uint2 r = make_uint2(xr | (min(w, 0xFFFFu) << 16),
+                               min(f[e].y, 0x7FFFFFFFu) | (q % 3ull == 0ull ? 0x80000000u : 0u));
+    s_rec[j0 + e] = r;
+    rec[j0 + e] = r;
+    P += w;
+  }
+  uint32_t at = block_scan_incl<uint32_t>(cnt, ws, &tot) - cnt;
+#pragma unroll
+  for (int e = 0; e < kPer; ++e)
+    if ((starts >> e) & 1u) s_sg[1u + at++] = (uint16_t)(j0 + e);
+  if (tid == 0) {
+    s_sg[0] = (uint16_t)tot;
+    s_sg[1u + tot] = (uint16_t)C;
+  }
+  return block_max<uint32_t>(mo, ws);
+}
+
 // smem_raw: push_smem_bytes(a.front_cap) bytes of shared memory (128-byte aligned).
 // NT: threads of the CTA (a power of two, 64 .. 1024).
 template <int NT>
@@ -625,7 +717,13 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
   } else if (C > p.max_boxes) {
     status = FA_E_CAPACITY;
   } else {
-    Om = om + over;
+    const bool one = C > 0u && C <= kChunk;  // one chunk: scanned here
+    uint32_t m = over;
+    if (one)
+      m = scan_one_chunk<NT>(p.fs, p.rec8 + (size_t)kidx * p.max_chunks * kChunk, C, kidx, a.shift, a.min_box, a.gutter,
+                             a.atlas_log2, reinterpret_cast<uint2*>(smem_raw),
+                             reinterpret_cast<uint16_t*>(smem_raw + kChunk * 8u));
+    Om = om + m;
     if (Om > a.front_cap) {
       status = FA_E_CAPACITY;
     } else {
@@ -648,6 +746,10 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
         mbar_init(&s_bar[1], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        if (one) {  // its stage is filled: complete the barrier's phase without a copy
+          mbar_expect_tx(&s_bar[0], 0u);
+          issued = 1;
+        }
         for (; issued < nchunks && issued < 2u; ++issued) issue(issued);
       }
       __syncthreads();

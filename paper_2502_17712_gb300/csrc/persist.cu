@@ -173,7 +173,7 @@ __device__ __noinline__ void st_bbox(const ViewArgs& v, uint32_t j, uint32_t n) 
   pm::bbox_body<DEV_M>(v.box, j, n);
 }
 __device__ __noinline__ void st_order_tile(const ViewArgs& v, uint32_t j, unsigned char* smem) {
-  pk::order_tile_body<true>(v.ps, v.fb, v.foot, j, reinterpret_cast<uint32_t*>(smem));
+  pk::order_tile_body<true>(v.ps, v.fa, v.fb, v.foot, v.order, j, reinterpret_cast<uint32_t*>(smem));
 }
 __device__ __noinline__ void st_order_scatter(const ViewArgs& v, uint32_t j, unsigned char* smem) {
   pk::order_scatter_body(v.ps, v.fa, v.fb, v.order, j, reinterpret_cast<uint32_t*>(smem));
