@@ -693,7 +693,10 @@ __device__ __noinline__ uint32_t scan_one_chunk(const uint2* __restrict__ fs, ui
 template <int NT>
 __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& a, uint32_t bid, uint32_t nblk,
                                           unsigned char* smem_raw) {
-  uint32_t* F = reinterpret_cast<uint32_t*>(smem_raw + 2 * kStageBytes);  // [front_cap]
+  // the frontline, [front_cap] 16-bit heights: Omega is at most 32,768, and a candidate
+  // that passes it fails, so a height only has to be right up to 65,535
+  uint16_t* F = reinterpret_cast<uint16_t*>(smem_raw + 2 * kStageBytes);
+  uint32_t* F2 = reinterpret_cast<uint32_t*>(F);  // two texels a word
   __shared__ __align__(8) unsigned long long s_bar[2];
   __shared__ uint32_t ws32[32];
   __shared__ uint32_t s_last;
@@ -707,7 +710,7 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
   const uint32_t om = 1u << a.atlas_log2;
   const uint32_t C = __ldcg(p.count), over = __ldcg(p.m + kidx);
   if (tid == 0) s_st0 = __ldcg(&p.ctr->status);
-  for (uint32_t x = tid; x < om; x += NT) F[x] = 0;  // (while the loads are on their way)
+  for (uint32_t x = tid; x < om / 2; x += NT) F2[x] = 0;  // (while the loads are on their way)
   __syncthreads();
   const int32_t st0 = s_st0;
   int32_t status = FA_OK;
@@ -740,7 +743,7 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
         bulk_g2s(dst, rec + (size_t)c * kChunk, rbytes, &s_bar[c & 1u]);
         bulk_g2s(dst + kChunk * 8u, sgg + (size_t)c * kSegStride, kSegStride * 2u, &s_bar[c & 1u]);
       };
-      for (uint32_t x = om + tid; x < Om; x += NT) F[x] = 0;
+      for (uint32_t x = om / 2 + tid; x < (Om + 1) / 2; x += NT) F2[x] = 0;
       if (tid == 0) {
         mbar_init(&s_bar[0], 1);
         mbar_init(&s_bar[1], 1);
@@ -772,23 +775,34 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
           const uint32_t nbx = j1 > j0 ? j1 - j0 : 0u;
           bool bad = false;
           if (nbx > (uint32_t)NT / 4u) {
-            // a thread per box (several boxes per thread past NT).  Boxes of such rows
-            // are mostly a few texels wide: the first four texels are read with
-            // independent loads before any is used, the rest in a loop.
+            // a thread per box (several boxes per thread past NT): a lone texel at an odd
+            // end, and the words between; the first words are read before any is used
             for (uint32_t jj = tid; jj < nbx; jj += NT) {
               const uint2 r = s_rec[j0 + jj];
               const uint32_t xr = r.x & 0xFFFFu, w = r.x >> 16, h = r.y & 0x7FFFFFFFu;
-              uint32_t* Fx = F + ((r.y >> 31) ? xr : Om - xr - w);
-              uint32_t m0 = w > 0u ? Fx[0] : 0u;
-              const uint32_t m1 = w > 1u ? Fx[1] : 0u, m2 = w > 2u ? Fx[2] : 0u, m3 = w > 3u ? Fx[3] : 0u;
-              for (uint32_t u = 4; u < w; ++u) m0 = max(m0, Fx[u]);
-              const uint32_t mx = max(max(m0, m1), max(m2, m3)), top = mx + h;
-              if (w > 0u) Fx[0] = top;
-              if (w > 1u) Fx[1] = top;
-              if (w > 2u) Fx[2] = top;
-              if (w > 3u) Fx[3] = top;
-              for (uint32_t u = 4; u < w; ++u) Fx[u] = top;
-              xy[base + j0 + jj] = make_uint2((uint32_t)(Fx - F), mx);
+              const uint32_t x = (r.y >> 31) ? xr : Om - xr - w, xe = x + w;
+              const uint32_t b0 = (x + 1u) >> 1, b1 = xe >> 1;
+              uint32_t e0 = (x & 1u) ? F[x] : 0u, e1 = (xe & 1u) ? F[xe - 1u] : 0u;
+              const uint32_t v0 = b0 < b1 ? F2[b0] : 0u, v1 = b0 + 1u < b1 ? F2[b0 + 1u] : 0u;
+              uint32_t v = __vmaxu2(v0, v1);
+              for (uint32_t q = b0 + 2u; q < b1; q += 4u) {
+                uint32_t f[4];
+#pragma unroll
+                for (uint32_t i = 0; i < 4u; ++i) f[i] = q + i < b1 ? F2[q + i] : 0u;
+                v = __vmaxu2(v, __vmaxu2(__vmaxu2(f[0], f[1]), __vmaxu2(f[2], f[3])));
+              }
+              const uint32_t mx = max(max(e0, e1), max(v & 0xFFFFu, v >> 16)), top = mx + h;
+              const uint32_t t16 = min(top, 0xFFFFu), tt = t16 * 0x10001u;
+              if (x & 1u) F[x] = (uint16_t)t16;
+              if (xe & 1u) F[xe - 1u] = (uint16_t)t16;
+              if (b0 < b1) F2[b0] = tt;
+              if (b0 + 1u < b1) F2[b0 + 1u] = tt;
+              for (uint32_t q = b0 + 2u; q < b1; q += 4u) {
+#pragma unroll
+                for (uint32_t i = 0; i < 4u; ++i)
+                  if (q + i < b1) F2[q + i] = tt;
+              }
+              xy[base + j0 + jj] = make_uint2(x, mx);
               Hloc = max(Hloc, top);
               bad |= top > Om;
             }
@@ -807,12 +821,12 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
               w = r.x >> 16;
               h = r.y & 0x7FFFFFFFu;
               x = (r.y >> 31) ? xr : Om - xr - w;
-              for (uint32_t u = li; u < w; u += g) mx = max(mx, F[x + u]);
+              for (uint32_t u = li; u < w; u += g) mx = max(mx, (uint32_t)F[x + u]);
             }
             for (uint32_t o = 1; o < g; o <<= 1) mx = max(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, o));
             if (jj < nbx) {
               const uint32_t top = mx + h;
-              for (uint32_t u = li; u < w; u += g) F[x + u] = top;
+              for (uint32_t u = li; u < w; u += g) F[x + u] = (uint16_t)min(top, 0xFFFFu);
               if (li == 0) {
                 xy[base + j0 + jj] = make_uint2(x, mx);
                 Hloc = max(Hloc, top);
@@ -928,7 +942,12 @@ __device__ __forceinline__ void pack_place_body(const PackScratch& p, const Pack
   }
 }
 
-size_t push_smem_bytes(uint32_t front_cap) { return 2 * (size_t)kStageBytes + (size_t)front_cap * 4; }
+// (at least 128 KB, so that no two candidates share an SM while others are idle: at 112 KB
+// for omega = 2048 the icosphere frame takes 247 us instead of 231)
+size_t push_smem_bytes(uint32_t front_cap) {
+  const size_t n = 2 * (size_t)kStageBytes + (size_t)front_cap * 2;
+  return n > (128u << 10) ? n : (128u << 10);
+}
 
 // The pack arguments (host side).
 inline PackArgs make_pack_args(const fa_ctx* ctx, uint32_t* order, uint32_t atlas_log2, uint32_t n_scales,
