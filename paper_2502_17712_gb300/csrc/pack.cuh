@@ -690,12 +690,13 @@ __device__ __noinline__ uint32_t scan_one_chunk(const uint2* __restrict__ fs, ui
 
 // smem_raw: push_smem_bytes(a.front_cap) bytes of shared memory (128-byte aligned).
 // NT: threads of the CTA (a power of two, 64 .. 1024).
-template <int NT>
+// STAGES: chunks in flight (1 or 2).
+template <int NT, uint32_t STAGES = 2>
 __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& a, uint32_t bid, uint32_t nblk,
                                           unsigned char* smem_raw) {
   // the frontline, [front_cap] 16-bit heights: Omega is at most 32,768, and a candidate
   // that passes it fails, so a height only has to be right up to 65,535
-  uint16_t* F = reinterpret_cast<uint16_t*>(smem_raw + 2 * kStageBytes);
+  uint16_t* F = reinterpret_cast<uint16_t*>(smem_raw + STAGES * kStageBytes);
   uint32_t* F2 = reinterpret_cast<uint32_t*>(F);  // two texels a word
   __shared__ __align__(8) unsigned long long s_bar[2];
   __shared__ uint32_t ws32[32];
@@ -736,12 +737,12 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
       const uint32_t nchunks = (C + kChunk - 1) / kChunk;
       uint32_t issued = 0;  // chunks whose copies were issued (thread 0)
       auto issue = [&](uint32_t c) {
-        unsigned char* dst = smem_raw + (c & 1u) * kStageBytes;
+        unsigned char* dst = smem_raw + (c % STAGES) * kStageBytes;
         const uint32_t nb = min(C - c * kChunk, kChunk);
         const uint32_t rbytes = ((nb + 1u) & ~1u) * 8u;  // whole 16-byte units (padded chunk)
-        mbar_expect_tx(&s_bar[c & 1u], rbytes + kSegStride * 2u);
-        bulk_g2s(dst, rec + (size_t)c * kChunk, rbytes, &s_bar[c & 1u]);
-        bulk_g2s(dst + kChunk * 8u, sgg + (size_t)c * kSegStride, kSegStride * 2u, &s_bar[c & 1u]);
+        mbar_expect_tx(&s_bar[c % STAGES], rbytes + kSegStride * 2u);
+        bulk_g2s(dst, rec + (size_t)c * kChunk, rbytes, &s_bar[c % STAGES]);
+        bulk_g2s(dst + kChunk * 8u, sgg + (size_t)c * kSegStride, kSegStride * 2u, &s_bar[c % STAGES]);
       };
       for (uint32_t x = om / 2 + tid; x < (Om + 1) / 2; x += NT) F2[x] = 0;
       if (tid == 0) {
@@ -753,14 +754,14 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
           mbar_expect_tx(&s_bar[0], 0u);
           issued = 1;
         }
-        for (; issued < nchunks && issued < 2u; ++issued) issue(issued);
+        for (; issued < nchunks && issued < STAGES; ++issued) issue(issued);
       }
       __syncthreads();
       uint32_t Hloc = 0, consumed = 0;
       bool fail = false, timed_out = false;
       for (uint32_t c = 0; c < nchunks; ++c) {
-        const uint32_t stg = c & 1u;
-        const bool got = mbar_wait_bounded(&s_bar[stg], (c >> 1) & 1u, a.wait_ns);
+        const uint32_t stg = c % STAGES;
+        const bool got = mbar_wait_bounded(&s_bar[stg], (c / STAGES) & 1u, a.wait_ns);
         if (__syncthreads_or(!got)) {
           timed_out = true;
           break;
@@ -854,7 +855,7 @@ __device__ __forceinline__ void push_body(const PackScratch& p, const PackArgs& 
       // copies still in flight land before the CTA leaves (with the full limit, also
       // after a time-out: the shared memory they write must outlive them)
       if (tid == 0)
-        for (uint32_t c = consumed; c < issued; ++c) mbar_wait_bounded(&s_bar[c & 1u], (c >> 1) & 1u, kWaitNs);
+        for (uint32_t c = consumed; c < issued; ++c) mbar_wait_bounded(&s_bar[c % STAGES], (c / STAGES) & 1u, kWaitNs);
       if (timed_out) {
         if (tid == 0) set_status(p.ctr, FA_E_TIMEOUT);
         status = FA_E_TIMEOUT;

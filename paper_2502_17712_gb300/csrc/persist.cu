@@ -182,7 +182,7 @@ __device__ __noinline__ void st_pack_scan(const ViewArgs& v, uint32_t j, uint32_
   pk::pack_scan_body<kPT, false>(v.ps, v.pa, v.n_scales, j, n);  // one candidate per item
 }
 __device__ __noinline__ void st_push(const ViewArgs& v, uint32_t j, uint32_t n, unsigned char* smem) {
-  pk::push_body<kPT>(v.ps, v.pa, j, n, smem);
+  pk::push_body<kPT, 1>(v.ps, v.pa, j, n, smem);
 }
 __device__ __noinline__ void st_place(const ViewArgs& v, uint32_t j, uint32_t n) { pk::pack_place_body(v.ps, v.pa, j, n); }
 template <bool DEV_M>
@@ -418,7 +418,9 @@ void build_view(fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params* p, cons
 }
 
 size_t persist_smem(uint32_t front_cap) {
-  return std::max<size_t>((size_t)kMaxH * 4u, pk::push_smem_bytes(front_cap));
+  // (one chunk staged at a time: 41 KB less than the push kernel, which the other
+  // stages' L1 gets)
+  return std::max<size_t>((size_t)kMaxH * 4u, pk::kStageBytes + (size_t)front_cap * 2u);
 }
 
 // Resident CTAs of the launch (one per SM at 1024 threads and this shared memory),
