@@ -65,16 +65,17 @@ template <bool LIST>
 __global__ void __launch_bounds__(kBlock) k_tri_chart(UfArgs a, const uint32_t* blockcnt, const uint2* wordroots,
                                                       int32_t* tri_chart, uint32_t* roots, uint32_t* box_enc,
                                                       uint32_t* box_full, uint32_t max_charts,
-                                                      const uint32_t* visstart, uint2* vis) {
+                                                      const uint32_t* visstart, uint2* vis, uint32_t tri_blocks,
+                                                      int32_t* vert_chart, int vertex_mode) {
   pdl_wait();
-  cf::tri_chart_body<LIST, kBlock>(a, blockcnt, wordroots, tri_chart, roots, box_enc, box_full, max_charts,
-                                   visstart, vis, blockIdx.x, gridDim.x);
-}
-
-__global__ void k_vert_chart(UfArgs a, const uint32_t* blockcnt, const uint2* wordroots, int32_t* vert_chart,
-                             int vertex_mode) {
-  pdl_wait();
-  cf::vert_chart_body(a, blockcnt, wordroots, vert_chart, vertex_mode, blockIdx.x, gridDim.x);
+  // (the vertices' charts, when asked for, by the blocks past tri_blocks: they read what
+  // the triangles' do, and a launch of their own costs 5 us)
+  if (blockIdx.x < tri_blocks)
+    cf::tri_chart_body<LIST, kBlock>(a, blockcnt, wordroots, tri_chart, roots, box_enc, box_full, max_charts,
+                                     visstart, vis, blockIdx.x, tri_blocks);
+  else
+    cf::vert_chart_body(a, blockcnt, wordroots, vert_chart, vertex_mode, blockIdx.x - tri_blocks,
+                        gridDim.x - tri_blocks);
 }
 
 }  // namespace
@@ -114,18 +115,12 @@ fa_status launch_chartify(fa_ctx* ctx, const fa_mesh* mesh, const uint32_t* vt, 
   launch_k(k_scan_blocks, 1, 1024, 0, s, ctx->blockcnt, ctx->viscnt, nb ? nb : 1, ch->count, ctx->cfg.max_charts,
            ctx->ctr);
   mark(ctx, "k_tri_chart", s);
-  if (tile_list && tri_chart_cleared)
-    launch_k(k_tri_chart<true>, nb < 152u * 8u ? (nb ? nb : 1u) : 152u * 8u, kBlock, 0, s, a, ctx->blockcnt,
-             ctx->wordroots, tri_chart, ch->root, ctx->box_enc, ctx->box_full, ctx->cfg.max_charts, ctx->viscnt,
-             ctx->vis);
-  else
-    launch_k(k_tri_chart<false>, nb ? nb : 1, kBlock, 0, s, a, ctx->blockcnt, ctx->wordroots, tri_chart, ch->root,
-             ctx->box_enc, ctx->box_full, ctx->cfg.max_charts, ctx->viscnt, ctx->vis);
-  if (vert_chart) {
-    mark(ctx, "k_vert_chart", s);
-    launch_k(k_vert_chart, grid_for(mesh->V, 256, 152 * 8), 256, 0, s, a, ctx->blockcnt, ctx->wordroots,
-             vert_chart, vm);
-  }
+  const bool listed = tile_list && tri_chart_cleared;
+  const uint32_t tb = listed ? std::min(nb ? nb : 1u, 152u * 8u) : (nb ? nb : 1u);
+  const uint32_t vb = vert_chart ? grid_for(mesh->V, kBlock, 152 * 8) : 0u;
+  launch_k(listed ? k_tri_chart<true> : k_tri_chart<false>, tb + vb, kBlock, 0, s, a, ctx->blockcnt, ctx->wordroots,
+           tri_chart, ch->root, ctx->box_enc, ctx->box_full, ctx->cfg.max_charts, ctx->viscnt, ctx->vis, tb, vert_chart,
+           vm);
   FA_CUDA_TRY(cudaGetLastError());
   return FA_OK;
 }
