@@ -29,16 +29,31 @@ Mat4 to_mat(const float* m) {
   return M;
 }
 
-template <class T>
-fa_status alloc(T** p, size_t n) {
-  *p = nullptr;
-  if (n == 0) n = 1;
-  if (cudaMalloc((void**)p, n * sizeof(T)) != cudaSuccess) {
-    cudaGetLastError();
-    return FA_E_OUT_OF_MEMORY;
+// The scratch of a context is one allocation: its parts are asked for first, each at a
+// 256-byte boundary, then placed.  (37 cudaMalloc and cudaFree calls took most of the time
+// of creating and destroying a small context.)
+struct Arena {
+  static constexpr int kMax = 64;
+  void** at[kMax];
+  size_t off[kMax];
+  int n = 0;
+  size_t bytes = 0;
+  template <class T>
+  void part(T** p, size_t count) {
+    at[n] = reinterpret_cast<void**>(p);
+    off[n++] = bytes;
+    bytes += (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~size_t(255);
   }
-  return FA_OK;
-}
+  fa_status place(void** base) {
+    if (cudaMalloc(base, bytes) != cudaSuccess) {
+      cudaGetLastError();
+      *base = nullptr;
+      return FA_E_OUT_OF_MEMORY;
+    }
+    for (int i = 0; i < n; ++i) *at[i] = static_cast<unsigned char*>(*base) + off[i];
+    return FA_OK;
+  }
+};
 
 fa_status check_view(const fa_ctx* ctx, const float* M, uint32_t W, uint32_t H) {
   if (!M || W == 0 || H == 0 || W > ctx->cfg.max_width || H > ctx->cfg.max_height) return FA_E_INVALID_ARG;
@@ -93,13 +108,7 @@ void fa_destroy(fa_ctx* ctx) {
   cudaDeviceSynchronize();
   if (ctx->prof_on)
     for (int i = 0; i <= kMaxProf; ++i) cudaEventDestroy(ctx->prof_ev[i]);
-  const PackScratch& p = ctx->pack;
-  void* ptrs[] = {ctx->ctr, ctx->zbuf, ctx->ties, ctx->zmax, ctx->queue, ctx->tile_owner, ctx->cand, ctx->surv, ctx->surv_count, ctx->surv_clip, ctx->clip, ctx->clip_count,
-                  ctx->label, ctx->wordroots, ctx->blockcnt, ctx->viscnt, ctx->vis, ctx->xedge, ctx->xcnt, ctx->tile_flag, ctx->tile_list,
-                  ctx->box_enc, ctx->box_full, p.ord_counts, p.ord_rank, p.ord_total,
-                  p.order, p.fs, p.rec8, p.segs, p.scan_state, p.m, p.xy, p.cand, ctx->psched};
-  for (void* p : ptrs)
-    if (p) cudaFree(p);
+  if (ctx->arena) cudaFree(ctx->arena);
   std::free(ctx);
 }
 
@@ -130,7 +139,6 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
   ctx->mid_max_pix = FA_RASTER_MID_OFF;
   ctx->uf_threads = 1024;
   ctx->push_threads = kDefaultPushThreads;
-  fa_status st = FA_OK;
   const uint64_t T = c.max_tris, V = c.max_verts, C = c.max_charts;
   ctx->queue_cap = (uint32_t)(T < (1u << 20) ? T + 1024 : (1u << 20));
   PackScratch& pk = ctx->pack;
@@ -138,50 +146,53 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
   pk.max_tiles = (uint32_t)((C + kOrderTile - 1) / kOrderTile);
   pk.max_chunks = (uint32_t)((C + kChunk - 1) / kChunk);
   const uint64_t nblocks = (T + 1023) / 1024 + 1;
-#define FA_ALLOC(ptr, n) \
-  if (st == FA_OK) st = alloc(&ptr, (size_t)(n));
-  FA_ALLOC(ctx->ctr, 1);
-  FA_ALLOC(ctx->zbuf, 2ull * c.max_width * c.max_height);
-  ctx->tie_cap = (uint32_t)std::max<uint64_t>(4096u, (uint64_t)c.max_width * c.max_height);
-  FA_ALLOC(ctx->ties, ctx->tie_cap);
-  FA_ALLOC(ctx->zmax, (uint64_t)((c.max_width + 15) / 16) * ((c.max_height + 15) / 16));
-  FA_ALLOC(ctx->queue, ctx->queue_cap);
+  Arena arena;
+  arena.part(&ctx->ctr, (size_t)(1));
+  arena.part(&ctx->zbuf, (size_t)(2ull * c.max_width * c.max_height));
+  arena.part(&ctx->zmax, (size_t)((uint64_t)((c.max_width + 15) / 16) * ((c.max_height + 15) / 16)));
+  arena.part(&ctx->queue, (size_t)(ctx->queue_cap));
   ctx->tile_cap = 4u * ctx->queue_cap;
-  FA_ALLOC(ctx->tile_owner, ctx->tile_cap);
-  // survivor regions (one per raster front block, each rounded up to 512 slots) and
-  // then the clipped-path candidate records
-  ctx->surv_cap = (uint32_t)(T + (uint64_t)fa::kMaxFrontBlocks * 512ull);
-  ctx->cand_cap = ctx->surv_cap + 65536u;
-  if (st == FA_OK) st = alloc((unsigned char**)&ctx->cand, (size_t)ctx->cand_cap * 48);
-  FA_ALLOC(ctx->surv, ctx->surv_cap);
-  FA_ALLOC(ctx->surv_count, fa::kMaxFrontBlocks);
-  if (st == FA_OK) st = alloc((float4**)&ctx->surv_clip, (size_t)ctx->surv_cap * 3);
-  FA_ALLOC(ctx->clip, ctx->surv_cap);
-  FA_ALLOC(ctx->clip_count, fa::kMaxFrontBlocks);
-  FA_ALLOC(ctx->label, T + V);
-  FA_ALLOC(ctx->wordroots, (T + 31) / 32);
-  FA_ALLOC(ctx->blockcnt, nblocks + 1);
-  FA_ALLOC(ctx->viscnt, nblocks + 1);
-  FA_ALLOC(ctx->xedge, nblocks * 3072);
-  FA_ALLOC(ctx->xcnt, nblocks);
-  FA_ALLOC(ctx->tile_flag, nblocks);
-  FA_ALLOC(ctx->tile_list, nblocks);
-  FA_ALLOC(ctx->vis, T);
-  FA_ALLOC(ctx->box_enc, 4 * C);
-  FA_ALLOC(ctx->box_full, C);
-  FA_ALLOC(pk.ord_counts, (uint64_t)kMaxH * pk.max_tiles);
-  FA_ALLOC(pk.ord_rank, C);
-  FA_ALLOC(pk.ord_total, kMaxH);
-  FA_ALLOC(pk.order, C);
-  FA_ALLOC(pk.fs, (uint64_t)pk.max_chunks * kChunk);
-  FA_ALLOC(pk.rec8, (uint64_t)kMaxScales * pk.max_chunks * kChunk);
-  FA_ALLOC(pk.segs, (uint64_t)kMaxScales * pk.max_chunks * kSegStride);
-  FA_ALLOC(pk.scan_state, (uint64_t)kMaxScales * pk.max_chunks);
-  FA_ALLOC(pk.m, kMaxScales);
-  FA_ALLOC(pk.xy, (uint64_t)kMaxScales * C);
-  FA_ALLOC(pk.cand, kMaxScales);
-  FA_ALLOC(ctx->psched, kPschedWords);
-#undef FA_ALLOC
+  arena.part(&ctx->tile_owner, (size_t)(ctx->tile_cap));
+  // survivor regions: one per raster front block, each rounded up to the block's threads;
+  // candidate records: the exact pass's blocks rounded up likewise, then the clipped path's
+  ctx->surv_cap = (uint32_t)(T + (uint64_t)fa::kFrontSlack);
+  ctx->cand_cap = (uint32_t)(T + 152ull * 8 * 256 + 65536u);
+  arena.part((unsigned char**)&ctx->cand, (size_t)ctx->cand_cap * 48);
+  arena.part(&ctx->surv, (size_t)(ctx->surv_cap));
+  arena.part(&ctx->surv_count, (size_t)(fa::kMaxFrontBlocks));
+  arena.part((float4**)&ctx->surv_clip, (size_t)ctx->surv_cap * 3);
+  arena.part(&ctx->clip, (size_t)(ctx->surv_cap));
+  arena.part(&ctx->clip_count, (size_t)(fa::kMaxFrontBlocks));
+  arena.part(&ctx->label, (size_t)(T + V));
+  arena.part(&ctx->wordroots, (size_t)((T + 31) / 32));
+  arena.part(&ctx->blockcnt, (size_t)(nblocks + 1));
+  arena.part(&ctx->viscnt, (size_t)(nblocks + 1));
+  arena.part(&ctx->xcnt, (size_t)(nblocks));
+  arena.part(&ctx->tile_flag, (size_t)(nblocks));
+  arena.part(&ctx->tile_list, (size_t)(nblocks));
+  arena.part(&ctx->box_enc, (size_t)(4 * C));
+  arena.part(&ctx->box_full, (size_t)(C));
+  arena.part(&pk.ord_counts, (size_t)((uint64_t)kMaxH * pk.max_tiles));
+  arena.part(&pk.ord_rank, (size_t)(C));
+  arena.part(&pk.ord_total, (size_t)(kMaxH));
+  arena.part(&pk.order, (size_t)(C));
+  arena.part(&pk.fs, (size_t)((uint64_t)pk.max_chunks * kChunk));
+  arena.part(&pk.rec8, (size_t)((uint64_t)kMaxScales * pk.max_chunks * kChunk));
+  arena.part(&pk.segs, (size_t)((uint64_t)kMaxScales * pk.max_chunks * kSegStride));
+  arena.part(&pk.scan_state, (size_t)((uint64_t)kMaxScales * pk.max_chunks));
+  arena.part(&pk.m, (size_t)(kMaxScales));
+  arena.part(&pk.xy, (size_t)((uint64_t)kMaxScales * C));
+  arena.part(&pk.cand, (size_t)(kMaxScales));
+  arena.part(&ctx->psched, (size_t)(kPschedWords));
+  fa_status st = arena.place(&ctx->arena);
+  if (st == FA_OK) {
+    // the chart passes' edges and visible list lie where the raster's clip coordinates
+    // were (last read by the marking pass), the raster's ties where the push records will be
+    ctx->xedge = static_cast<uint2*>(ctx->surv_clip);
+    ctx->vis = ctx->xedge + nblocks * 3072;
+    ctx->ties = reinterpret_cast<uint4*>(pk.rec8);
+    ctx->tie_cap = (uint32_t)((uint64_t)kMaxScales * pk.max_chunks * kChunk / 2);
+  }
   pk.ctr = ctx->ctr;
   pk.count = nullptr;
   if (st == FA_OK && cudaMemset(ctx->ctr, 0, sizeof(DevCounters)) != cudaSuccess) st = FA_E_CUDA;

@@ -32,6 +32,7 @@ constexpr unsigned long long kWaitNs = FA_DEFAULT_WAIT_NS;  // device time limit
 
 // Small counters that live in device memory (one struct per context).
 constexpr uint32_t kMaxFrontBlocks = 152 * 4;  // raster front-end blocks (survivor regions)
+constexpr uint32_t kFrontSlack = 152 * 1024;   // their threads at most (a region holds whole rounds of its block)
 constexpr uint32_t kDefaultPushThreads = 512;  // threads of a candidate's push CTA (fa_set_chart_pack_schedule)
 constexpr uint32_t kPschedWords = 64;          // schedule state of a single-view persistent launch
 
@@ -115,10 +116,11 @@ struct fa_ctx {
   int prof_n;
   cudaEvent_t prof_ev[kMaxProf + 1];
   const char* prof_name[kMaxProf];
-  // scratch
+  // scratch, all of it in one allocation
+  void* arena;
   fa::DevCounters* ctr;
   uint32_t* zbuf;        // [max_w * max_h] depth keys, or 64-bit key | triangle
-  uint4* ties;           // [tie_cap] pixels where two triangles have the same key
+  uint4* ties;           // [tie_cap] pixels where two triangles have the same key (in pack.rec8)
   uint32_t tie_cap;
   uint32_t* zmax;        // [ceil(max_w / 16) * ceil(max_h / 16)] largest depth key per 16x16 tile
   uint32_t* tile_flag;   // [ceil(max_tris / 1024)] tile has a visible triangle (this frame)
@@ -138,10 +140,10 @@ struct fa_ctx {
   int32_t* label;        // [max_tris + max_verts]
   uint2* wordroots;      // [ceil(max_tris / 32)] per VT word: root bits, roots before it in its block
   uint32_t* blockcnt;    // [n_blocks + 1]
-  uint2* xedge;          // [n_blocks][3072] cross-tile edges of the local union-find
+  uint2* xedge;          // [n_blocks][3072] cross-tile edges of the local union-find (in surv_clip)
   uint32_t* xcnt;        // [n_blocks] their counts
   uint32_t* viscnt;      // [n_blocks + 1] visible triangles per 1024-triangle block, then their starts
-  uint2* vis;            // [max_tris] (triangle, chart) of the visible triangles, triangle order
+  uint2* vis;            // [max_tris] (triangle, chart) of the visible triangles, triangle order (in surv_clip)
   uint32_t* box_enc;     // [max_charts * 4] ordered-int chart boxes
   uint32_t* box_full;    // [max_charts]
   fa::PackScratch pack;  // order + pack scratch (count filled per call)

@@ -341,7 +341,7 @@ void build_view(fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params* p, cons
   const uint64_t chart_cap = std::min<uint64_t>(ctx->cfg.max_charts, T);
   const uint32_t ntiles = (T + 1023) / 1024;
   const uint64_t pix = (uint64_t)W * H;
-  const uint32_t n_front = std::min<uint32_t>(wk(T, 128), kMaxFrontBlocks);
+  const uint32_t n_front = std::min<uint32_t>(wk(T, 128), kFrontSlack / kPT);
   const uint32_t n_tri = wk(T, 128);
   const uint32_t n_pix = wk(pix, 2048);
   const uint32_t n_tiles = clampu(ntiles, 1, G);

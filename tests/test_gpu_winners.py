@@ -28,16 +28,19 @@ def visible(F, pos, idx, M, W, H, flags=0):  # noqa: F811
     return out
 
 
-@pytest.mark.parametrize("copies", [1, 2, 5])  # 5: more ties than the list holds (64 * 64)
-@pytest.mark.parametrize("n,radius", [(64, 1.6), (9, 1.6), (2, 1.6), (2, 0.3)])  # small, mid-size, large, clipped
+@pytest.mark.parametrize("copies", [1, 2, 5])  # 5: more ties than the list holds (131,072)
+@pytest.mark.parametrize("n,radius", [(200, 1.6), (40, 1.6), (2, 1.6), (2, 0.3)])  # small, mid-size, large, clipped
 def test_coplanar_stacks(F, copies, n, radius):  # noqa: F811
     """Copies of one patch at the same place: every copy of a visible triangle is visible."""
     sc = S.grid_scene(5, n)
     pos = np.concatenate([sc.pos] * copies)
     idx = np.concatenate([sc.idx + np.uint32(c * sc.V) for c in range(copies)])
-    M = S.view_proj((0.1, -0.2, radius), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), 64, 64)
-    vt = visible(F, pos, idx, M, 64, 64)
-    want = O.visibility(M, pos, idx, 64, 64)
+    W = H = 400
+    M = S.view_proj((0.1, -0.2, radius), (0.0, 0.0, 0.0), (0.0, 1.0, 0.0), W, H)
+    vt = visible(F, pos, idx, M, W, H)
+    want, z = O.visibility(M, pos, idx, W, H, return_zbuf=True)
+    covered = int((z != 0xFFFFFFFF).sum())
+    assert copies < 5 or (copies - 1) * covered > 131072
     assert want.any() and (vt == want).all()
 
 
