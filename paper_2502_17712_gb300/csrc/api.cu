@@ -357,7 +357,7 @@ fa_status enqueue_frame(fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params*
   // pass then writes only the listed tiles
   const bool tri_init = (reinterpret_cast<uintptr_t>(o->tri_chart) & 15u) == 0;
   if ((st = launch_visibility(ctx, mesh, M, p->width, p->height, o->vt, true, s, Md,
-                              (p->flags & FA_VIS_CONSERVATIVE) != 0, tri_init ? o->tri_chart : nullptr)) != FA_OK)
+                              (p->flags & FA_VIS_CONSERVATIVE) != 0, tri_init ? o->tri_chart : nullptr, o->partial)) != FA_OK)
     return st;
   if ((st = launch_chartify(ctx, mesh, o->vt, p->chart_mode, o->tri_chart, o->vert_chart, &o->charts, s,
                             true, tri_init)) != FA_OK)

@@ -377,7 +377,7 @@ inline void launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
 fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W,
                             uint32_t H, uint32_t* vt, bool reset_status, cudaStream_t s,
                             const float* Mdev = nullptr, bool conservative = false,
-                            int32_t* tri_chart_init = nullptr);
+                            int32_t* tri_chart_init = nullptr, uint32_t* partial_clear = nullptr);
 // tile_list: the marking pass of the same frame listed the tiles with a visible
 // triangle (and the raster front end zeroed the per-tile counts and set tri_chart
 // to -1), so the union-find and chart-id passes visit only those

@@ -57,7 +57,9 @@ fa_status launch_parameterize(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, u
                               float ratio, const int32_t* tri_chart, const fa_charts* ch, bool reset_boxes,
                               uint32_t flags, uint32_t* partial, cudaStream_t s, const float* Mdev,
                               bool footprint, bool listed) {
-  if (partial) FA_CUDA_TRY(cudaMemsetAsync(partial, 0, (size_t)((mesh->T + 31) / 32) * 4, s));
+  // (on the frame path the raster front end has cleared the bits: a memset between the
+  // kernels would also end their programmatic launch there)
+  if (partial && reset_boxes) FA_CUDA_TRY(cudaMemsetAsync(partial, 0, (size_t)((mesh->T + 31) / 32) * 4, s));
   if (reset_boxes) {
     mark(ctx, "k_box_reset", s);
     launch_k(k_box_reset, grid_for(ctx->cfg.max_charts, 256, 152 * 4), 256, 0, s, ch->count, ctx->cfg.max_charts,

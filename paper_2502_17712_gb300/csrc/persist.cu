@@ -32,11 +32,11 @@ namespace fa {
 namespace {
 
 constexpr int kPT = 1024;           // threads per CTA
-constexpr int kMaxStages = 24;      // stages of one view (at most 20 are used)
+constexpr int kMaxStages = 24;      // stages of one view (at most 21 are used)
 constexpr int kInlineGroups = 24;   // stage groups of a single-view launch (kernel parameter)
 
 enum Stage : uint8_t {
-  S_FRONT, S_EXACT, S_DEPTH_BIG, S_ZMAX, S_MARK, S_INIT_V, S_LOCAL, S_HOOK, S_HOOK_V, S_HOOK_NM, S_FLATTEN, S_SCAN,
+  S_FRONT, S_EXACT, S_DEPTH_BIG, S_ZMAX, S_MARK, S_MARK_CONS, S_INIT_V, S_LOCAL, S_HOOK, S_HOOK_V, S_HOOK_NM, S_FLATTEN, S_SCAN,
   S_TRI_CHART, S_VERT_CHART, S_BBOX, S_ORDER_TILE, S_ORDER_SCATTER, S_PACK_SCAN, S_PUSH, S_PLACE, S_UV
 };
 
@@ -140,6 +140,9 @@ __device__ __noinline__ void st_mark(const ViewArgs& v, uint32_t j, uint32_t n) 
 __device__ __noinline__ void st_mark_win(const ViewArgs& v, uint32_t j, uint32_t n) {
   rs::mark_win_body<kPT>(v.ra, j, n);
 }
+__device__ __noinline__ void st_mark_cons(const ViewArgs& v, uint32_t j, uint32_t n) {
+  rs::mark_cons_body<kPT>(v.ra, j, n);
+}
 __device__ __noinline__ void st_init_v(const ViewArgs& v, uint32_t j, uint32_t n) {
   cf::init_v_body(v.uf.label, v.uf.T, v.uf.V, j, n);
 }
@@ -215,6 +218,7 @@ __device__ void run_stage(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_
     case S_DEPTH_BIG: v.ra.win ? st_depth_win(v, j, n) : st_depth_big(v, j, n); break;
     case S_ZMAX: st_zmax(v, j, n); break;
     case S_MARK: v.ra.win ? st_mark_win(v, j, n) : v.cons ? st_mark<true>(v, j, n) : st_mark<false>(v, j, n); break;
+    case S_MARK_CONS: st_mark_cons(v, j, n); break;
     case S_INIT_V: st_init_v(v, j, n); break;
     case S_LOCAL: st_local(v, j, n); break;
     case S_HOOK: st_hook(v, j, n); break;
@@ -399,6 +403,7 @@ void build_view(fa_ctx* ctx, const fa_mesh* mesh, const fa_frame_params* p, cons
   add(S_DEPTH_BIG, n_pix);
   if (v.ra.zmax) add(S_ZMAX, wk(pix, 8192));
   add(S_MARK, std::max(n_rast, n_pix));
+  if (v.cons) add(S_MARK_CONS, n_rast);  // (nothing to do with the tile-depth option on)
   if (vm) add(S_INIT_V, wk(mesh->V, 128));
   add(S_LOCAL, n_tiles);
   add(vm ? S_HOOK_V : S_HOOK, vm ? n_tri : clampu((ntiles + 7) / 8, 1, G));

@@ -46,11 +46,16 @@ __global__ void __launch_bounds__(256, 4) k_raster_mark(RasterArgs A) {
   else rs::mark_body<MODE == kMarkConservative, 256>(A, blockIdx.x, gridDim.x);
 }
 
+__global__ void __launch_bounds__(256, 4) k_raster_mark_cons(RasterArgs A) {
+  pdl_wait();
+  rs::mark_cons_body<256>(A, blockIdx.x, gridDim.x);
+}
+
 }  // namespace
 
 fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uint32_t W, uint32_t H,
                             uint32_t* vt, bool reset_status, cudaStream_t s, const float* Mdev, bool cons,
-                            int32_t* tri_chart_init) {
+                            int32_t* tri_chart_init, uint32_t* partial_clear) {
   // one wave (two resident blocks per SM): half the survivor regions of two waves,
   // so the passes that look regions up scan fewer counts
   // (and enough blocks for the clears: at most 16 depth-buffer pixels per thread)
@@ -59,6 +64,7 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
   const unsigned gb = 152 * 8;
   RasterArgs A = rs::make_raster_args(ctx, mesh, M, W, H, vt, reset_status, Mdev, cons, tri_chart_init, fb,
                                             rs::kFrontThreads);
+  A.partial_clear = partial_clear;
   rs::set_exact_grid(A, gb, 256);
   ctx->front_blocks = A.front_blocks;
   mark(ctx, "k_raster_front", s);
@@ -83,6 +89,10 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
     launch_k(k_raster_mark<kMarkWinners>, std::min(((W + 63) / 64) * ((H + 31) / 32), 152u * 8u), 256, 0, s, A);
   else
     launch_k(cons ? k_raster_mark<kMarkConservative> : k_raster_mark<kMarkSamples>, 152 * 4, 256, 0, s, A);
+  if (A.win && cons) {
+    mark(ctx, "k_raster_mark_cons", s);
+    launch_k(k_raster_mark_cons, 152 * 8, 256, 0, s, A);
+  }
   FA_CUDA_TRY(cudaGetLastError());
   return FA_OK;
 }

@@ -1752,6 +1752,126 @@ __device__ __forceinline__ void mark_win_body(const RasterArgs& A, uint32_t bid,
   }
 }
 
+// Conservative marking after the winners': the triangles that the samples marked are
+// marked already (a covered centre's depth is the sample's), so only the other survivors
+// are tested, each pixel of their conservative boxes against the final keys (as
+// sample<2>).  With many survivors, boxes of at most kSmallMaxPix pixels in-thread and
+// larger ones by the warp together; with few, a warp takes few of them, all together.
+// Against a second rasterization of every survivor (conservative fa_visibility at 1080p):
+// a floor of 60 patches 387 -> 250 us, 200 icospheres 209 -> 183.  What is left is the
+// hidden triangles' boxes, every pixel of them; four pixels' loads at once cost
+// registers and are slower (321, 206).
+__device__ __forceinline__ bool cons_box(const RasterArgs& A, const SV& a, const SV& b, const SV& c, int px0, int py0,
+                                         int px1, int py1, uint32_t first, uint32_t step) {
+  const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
+  const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
+  const float zmin = fminf(a.zn, fminf(b.zn, c.zn)), zmax = fmaxf(a.zn, fmaxf(b.zn, c.zn));
+  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
+  for (uint32_t s = first; s < n; s += step) {
+    const int px = px0 + (int)(s % w), py = py0 + (int)(s / w);
+    const Edges E = edges_at(a, b, c, px, py);
+    bool meets = true, in = true;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const int64_t ax = E.dx[i] < 0 ? -E.dx[i] : E.dx[i], ay = E.dy[i] < 0 ? -E.dy[i] : E.dy[i];
+      meets = meets && E.e[i] + ((ax + ay) >> 1) >= 0;
+      in = in && (E.e[i] > 0 || (E.e[i] == 0 && E.tl[i]));
+    }
+    if (!meets) continue;
+    float f = __fmul_rn(ll2float_rn(E.e[0]), a.zn);
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[1]), b.zn));
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[2]), c.zn));
+    float d = __fmul_rn(f, invA);
+    if (!in) d = fminf(fmaxf(d, zmin), zmax);
+    if (!(d >= -1.0f && d <= 1.0f)) continue;
+    if (ordered(d) <= zkey(A, (uint32_t)py * (uint32_t)A.W + (uint32_t)px)) return true;
+  }
+  return false;
+}
+
+// The sub-triangles of a triangle that must be clipped (rare).
+__device__ __noinline__ bool cons_clipped(const RasterArgs& A, float4 c0, float4 c1, float4 c2) {
+  CV poly[kMaxPoly];
+  poly[0] = CV{c0.x, c0.y, c0.z, c0.w};
+  poly[1] = CV{c1.x, c1.y, c1.z, c1.w};
+  poly[2] = CV{c2.x, c2.y, c2.z, c2.w};
+  const int n = clip_polygon(poly, 3);
+  if (n < 3) return false;
+  for (int i = 0; i < n; ++i)
+    if (!(poly[i].w > 0.0f)) return false;
+  SV sv[kMaxPoly];
+  for (int i = 0; i < n; ++i) sv[i] = project(poly[i], A.hx, A.hy);
+  for (int i = 1; i + 1 < n; ++i) {
+    const Setup s = setup(sv[0], sv[i], sv[i + 1], A.W, A.H, true);
+    if (s.A <= 0 || s.px1 < s.px0 || s.py1 < s.py0) continue;
+    if (cons_box(A, sv[0], sv[i], sv[i + 1], s.px0, s.py0, s.px1, s.py1, 0u, 1u)) return true;
+  }
+  return false;
+}
+
+template <int NT>
+__device__ __forceinline__ void mark_cons_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  if (!A.win || !A.cons) return;
+  uint32_t* pre = region_pre();
+  __shared__ int32_t s_cons_status;
+  if (threadIdx.x == 0) s_cons_status = __ldcg(&A.ctr->status);
+  __syncthreads();
+  if (s_cons_status != 0) return;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t n = surv_prefix<NT>(A, pre);
+  const uint32_t stride = nblk * blockDim.x, warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = stride >> 5;
+  uint32_t per = 32;  // survivors a warp takes at a time
+  while (per > 1u && (uint64_t)n * 32u <= (uint64_t)nwarps * per * 16u) per >>= 1;
+  for (uint32_t base = warp * per; base < n; base += nwarps * per) {
+    const uint32_t v = base + lane;
+    SV a{0, 0, 0.0f}, b{0, 0, 0.0f}, c{0, 0, 0.0f};
+    Setup S{0, 0, 0, -1, -1};
+    uint32_t t = 0;
+    bool vis = false, big = false;
+    if (lane < per && v < n) {
+      const uint32_t i = surv_slot(A, pre, v, base);
+      t = __ldcg(A.surv + i);
+      if (!((__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u)) {
+        const float4* sc = A.surv_clip + 3 * (size_t)i;
+        const float4 c0 = __ldcs(sc), c1 = __ldcs(sc + 1), c2 = __ldcs(sc + 2);
+        a = project(CV{c0.x, c0.y, c0.z, c0.w}, A.hx, A.hy);
+        b = project(CV{c1.x, c1.y, c1.z, c1.w}, A.hx, A.hy);
+        c = project(CV{c2.x, c2.y, c2.z, c2.w}, A.hx, A.hy);
+        S = setup(a, b, c, A.W, A.H, true);
+        if (S.A > 0 && S.px1 >= S.px0 && S.py1 >= S.py0) {
+          big = (S.px1 - S.px0 + 1) * (S.py1 - S.py0 + 1) > (per < 32u ? 1 : kSmallMaxPix);
+          if (!big) vis = cons_box(A, a, b, c, S.px0, S.py0, S.px1, S.py1, 0u, 1u);
+        }
+      }
+    }
+    for (uint32_t m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1u) {  // the warp together
+      const int src = __ffs(m) - 1;
+      const SV qa{__shfl_sync(0xFFFFFFFFu, (int32_t)a.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)a.Y, src),
+                  __shfl_sync(0xFFFFFFFFu, a.zn, src)};
+      const SV qb{__shfl_sync(0xFFFFFFFFu, (int32_t)b.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)b.Y, src),
+                  __shfl_sync(0xFFFFFFFFu, b.zn, src)};
+      const SV qc{__shfl_sync(0xFFFFFFFFu, (int32_t)c.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)c.Y, src),
+                  __shfl_sync(0xFFFFFFFFu, c.zn, src)};
+      const int px0 = __shfl_sync(0xFFFFFFFFu, S.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, S.py0, src);
+      const int px1 = __shfl_sync(0xFFFFFFFFu, S.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, S.py1, src);
+      const bool hit = cons_box(A, qa, qb, qc, px0, py0, px1, py1, lane, 32u);
+      if (__any_sync(0xFFFFFFFFu, hit) && (int)lane == src) vis = true;
+    }
+    if (vis) win_mark(A, t);
+  }
+  __syncthreads();  // pre is reused
+  const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
+  const Mat4 M = A.Mdev ? load_mat(A.Mdev) : A.M;
+  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
+    const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
+    if ((__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u) continue;
+    const uint32_t* f = A.idx + 3 * (size_t)t;
+    if (cons_clipped(A, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
+                     load_clip(M, A.pos, __ldg(f + 2))))
+      win_mark(A, t);
+  }
+}
+
 inline void set_raster_mode(RasterArgs& A);
 
 // The arguments of one visibility pass on ctx (host side).  front_blocks blocks of
@@ -1809,9 +1929,8 @@ inline RasterArgs make_raster_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4&
   return A;
 }
 
-// Conservative marking tests other samples than the depth pass takes, and the tile-depth
-// option belongs to the second rasterization: both keep it.
-inline void set_raster_mode(RasterArgs& A) { A.win = !A.cons && !A.zmax ? 1 : 0; }
+// The tile-depth option belongs to the second rasterization and keeps it.
+inline void set_raster_mode(RasterArgs& A) { A.win = A.zmax ? 0 : 1; }
 
 // The exact pass's grid (blocks of `threads` threads), from which the mid-size lists get
 // their shares: a block sees at most mid_per_block survivors.

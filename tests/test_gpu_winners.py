@@ -60,3 +60,25 @@ def test_equals_second_rasterization(F, parts, n, W, H, radius):  # noqa: F811
     M = S.hemisphere_camera(parts, W, H, radius=radius)
     a, b = visible(F, sc.pos, sc.idx, M, W, H), visible(F, sc.pos, sc.idx, M, W, H, F.FA_RASTER_HIZ)
     assert a.any() and (a == b).all()
+
+
+@pytest.mark.parametrize("parts,n,W,H,radius", [(1, 64, 480, 270, 3.0), (40, 33, 901, 613, 7.0), (8, 5, 640, 360, 3.0),
+                                                (30, 9, 333, 222, 0.8), (2, 150, 63, 31, 6.0)])
+def test_conservative_marking(F, parts, n, W, H, radius):  # noqa: F811
+    """Conservative marking of what the samples left: small boxes, the warp's, clipped ones, triangles without a
+    pixel centre; against the oracle, and against the second rasterization."""
+    import torch
+    sc = S.instanced_grid_scene(parts, parts, n, half=1.5)
+    M = S.hemisphere_camera(parts + 5, W, H, radius=radius)
+    want = O.visibility(M, sc.pos, sc.idx, W, H, conservative=True)
+    ctx = F.Context(max_tris=sc.T, max_verts=sc.V, max_charts=16, max_width=W, max_height=H)
+    mesh = F.Mesh(ctx, sc.pos, sc.idx)
+    vt = torch.zeros((sc.T + 31) // 32, dtype=torch.int32, device="cuda")
+    for flags in (0, F.FA_RASTER_HIZ):
+        ctx.set_raster_schedule(16, flags)
+        F.fa_visibility(ctx.handle, mesh.handle, M, W, H, vt, flags=F.FA_VIS_CONSERVATIVE)
+        torch.cuda.synchronize()
+        assert ctx.device_status() == F.FA_OK
+        assert want.any() and (vt.cpu().numpy().view(np.uint32) == want).all()
+    mesh.close()
+    ctx.close()
