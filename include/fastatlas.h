@@ -417,7 +417,7 @@ uint64_t fa_launch_count(const fa_ctx* ctx);
 typedef struct fa_frame_stats {
   uint32_t survivors;     /* triangles that passed the raster front end */
   uint32_t clipped;       /* of those, triangles that needed clipping */
-  uint32_t clip_records;  /* small sub-triangle records of the clipping path */
+  uint32_t clip_records;  /* small sub-triangle records of the clipping path (FA_RASTER_HIZ; else 0) */
   uint32_t big_entries;   /* large sub-triangles queued for tile rasterization */
   uint64_t big_tiles;     /* their 16x16 tiles */
   uint32_t visible;       /* entries of the visible-triangle list */

@@ -7,7 +7,8 @@
 //   1024-box tile stably inside their height bin (a shared-memory histogram the
 //   warps update in index order) and writes a per-bin count row per tile and the
 //   global bin totals; k_order_scatter scans the totals (every block) and adds, for
-//   each box, the counts of its bin in earlier tiles.
+//   each box, the counts of its bin in earlier tiles.  Boxes of one tile are put in
+//   order by k_order_tile alone.
 //   This replaces the paper's cuckoo-hash bucketing with the same result contract
 //   (deterministic, identical for identical frames).
 //
@@ -19,7 +20,8 @@
 //   row, w, h, row direction) plus per chunk the list of row segments.  Then one CTA
 //   per candidate (k_pack_push) pushes the rows up against a frontline in shared
 //   memory, with the chunks staged by bulk asynchronous copies; segments of one
-//   row never overlap in x, so a row may span two chunks.  The last CTA to finish
+//   row never overlap in x, so a row may span two chunks.  Boxes of one chunk are
+//   scanned by the candidates' own CTAs, not by k_pack_scan.  The last CTA to finish
 //   selects the candidate.  The placements are written by the UV kernel on the frame
 //   path and by k_pack_place (all CTAs) for a standalone packing.
 #pragma once
