@@ -357,9 +357,9 @@ fa_status fa_last_device_status(fa_ctx* ctx, fa_stream_t stream, int32_t* out);
 fa_status fa_set_wait_limits(fa_ctx* ctx, uint32_t loop_cap, uint64_t wait_ns);
 
 /* Raster schedule of this context's later frames (changes timing only, never
- * results).  By default a frame with sample-coverage marking is rasterized once (the
- * depth pass keeps each pixel's triangle); conservative marking and FA_RASTER_HIZ
- * rasterize a second time to mark, and mid_max_pix applies to them.
+ * results).  By default a frame is rasterized once (the depth pass keeps each pixel's
+ * triangle; conservative marking then tests what the samples left unmarked); with
+ * FA_RASTER_HIZ it is rasterized a second time to mark, and mid_max_pix applies then.
  *  mid_max_pix: a sub-triangle whose pixel box has at most 16 pixels is rasterized
  *    by one thread; larger ones are split into 16x16 tiles, one warp per tile.
  *    With mid_max_pix > 16, boxes of up to mid_max_pix pixels are also rasterized
@@ -368,12 +368,13 @@ fa_status fa_set_wait_limits(fa_ctx* ctx, uint32_t loop_cap, uint64_t wait_ns);
  *    views of many mid-size triangles (high resolutions, dense meshes seen close
  *    up); on views of mostly tiny triangles the tiles stay cheaper, hence the
  *    default FA_RASTER_MID_OFF.
- *  flags: FA_RASTER_HIZ adds a pass that takes the largest depth of every 16x16
- *    pixel tile of the final depth buffer; the marking pass then skips a
- *    sub-triangle (or a tile of one) whose smallest possible sample depth, less a
- *    bound on the depth's rounding error, is above the largest depth of every tile
- *    it touches.  That pays where most hidden triangles lie behind fully covered
- *    tiles (large overlapping surfaces); off by default.
+ *  flags: FA_RASTER_HIZ rasterizes twice and adds a pass that takes the largest
+ *    depth of every 16x16 pixel tile of the final depth buffer; the marking pass then
+ *    skips a sub-triangle (or a tile of one) whose smallest possible sample depth, less
+ *    a bound on the depth's rounding error, is above the largest depth of every tile it
+ *    touches.  Off by default: one rasterization is faster on every scene measured (64
+ *    views of overlapping floors one after the other: 17.5 ms, 27.2 with the option and
+ *    mid_max_pix 64).
  * Both ways the same samples get the same depth keys and the same triangles are
  * marked.  Errors: FA_E_INVALID_ARG (NULL ctx, mid_max_pix outside [16, 256],
  * unknown flags). */

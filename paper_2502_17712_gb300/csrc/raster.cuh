@@ -18,10 +18,11 @@
 // lanes each when the survivors are few for the grid), k_raster_depth_big (the larger
 // ones) and k_raster_mark (the visible bits; it also lists the 1024-triangle tiles
 // that hold a visible triangle for the chart passes).  Two forms of the last three:
-// "winners" (the default; below), where the depth pass keeps each pixel's triangle, and
-// two rasterizations (conservative marking, the tile-depth option), where the exact
-// pass keeps a 48-byte record of each small sub-triangle and the marking pass
-// rasterizes the queued tiles and the records again.  Edge values that stay below 2^24
+// "winners" (the default; below), where the depth pass keeps each pixel's triangle (with
+// conservative marking k_raster_mark_cons then tests what the samples left unmarked),
+// and two rasterizations (the tile-depth option), where the exact pass keeps a 48-byte
+// record of each small sub-triangle and the marking pass rasterizes the queued tiles and
+// the records again.  Edge values that stay below 2^24
 // over a box are there stepped as exact fp32 integers.
 #pragma once
 #include "fa_internal.cuh"
@@ -1075,7 +1076,7 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
 
 // ------------------------------------------------------------------ winners
 //
-// Single-pass visibility (sample-coverage marking; the default).  A sample of the
+// Single-pass visibility (the default).  A sample of the
 // marking pass passes "<=" exactly when its key equals the pixel's smallest key, and
 // both passes take the same samples, so the triangles to mark are those that own a
 // pixel's smallest key: the depth pass keeps key << 32 | triangle per pixel (64-bit
@@ -1088,11 +1089,12 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
 //
 // Three sizes of sub-triangles, so that the lanes of a warp have like work: boxes of at
 // most kSmallMaxPix pixels are rasterized where they are set up (exact pass); boxes of
-// at most kMidPix are listed and then rasterized by 1 .. 16 lanes each, as many as fill
-// the grid, a lane taking whole rows; larger ones are 16x16 tiles, a warp per tile.
-// Edge functions of sub-triangles of less than 96 pixels a side fit 32 bits (twice
-// the product of the sides is below 2^31, also 16 pixels past the box); their conversions to fp32 round as the 64-bit
-// ones do.  A top-left edge passes at 0, another one from 1, so that with 1 taken from
+// at most kMidPix are listed and then rasterized by 4 .. 32 lanes each, as many as fill
+// the grid, neighbouring lanes taking neighbouring samples; larger ones are 16x16 tiles,
+// a warp per tile.  Edge functions of sub-triangles of less than 96 pixels a side fit 32
+// bits (twice the product of the sides is 1.21e9; steps past the box's end, 128 rows of
+// one pixel at most, add 0.81e9); their conversions to fp32 round as the 64-bit ones do.
+// A top-left edge passes at 0, another one from 1, so that with 1 taken from
 // the others a sample is covered when no value is negative.
 //
 // What bounds it: the atomics' round trips and the instructions of the samples (the
