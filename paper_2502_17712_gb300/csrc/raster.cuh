@@ -1125,6 +1125,17 @@ struct WinSetup {
   bool live;  // front facing, with a sample in its box
 };
 
+__device__ __forceinline__ uint32_t tiles_of(int w, int h) {
+  return (uint32_t)((w + kBigTile - 1) / kBigTile) * (uint32_t)((h + kBigTile - 1) / kBigTile);
+}
+
+// 32-bit edge functions: the sides are short enough.
+__device__ __forceinline__ bool fits32(const Tri32& v) {
+  const int xmn = min(v.X[0], min(v.X[1], v.X[2])), xmx = max(v.X[0], max(v.X[1], v.X[2]));
+  const int ymn = min(v.Y[0], min(v.Y[1], v.Y[2])), ymx = max(v.Y[0], max(v.Y[1], v.Y[2]));
+  return xmx - xmn < kSpan32 && ymx - ymn < kSpan32;
+}
+
 __device__ __forceinline__ void project32(const float4& c, float hx, float hy, int& X, int& Y, float& z) {
   const SV s = project(CV{c.x, c.y, c.z, c.w}, hx, hy);
   X = (int)s.X;
@@ -1144,7 +1155,7 @@ __device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4&
   s.px1 = min((xmx - 128) >> 8, A.W - 1);
   s.py0 = max(-((128 - ymn) >> 8), 0);
   s.py1 = min((ymx - 128) >> 8, A.H - 1);
-  s.fits = xmx - xmn < kSpan32 && ymx - ymn < kSpan32;
+  s.fits = fits32(s.v);
   const int ux = s.v.X[1] - s.v.X[0], uy = s.v.Y[1] - s.v.Y[0], vx = s.v.X[2] - s.v.X[0], vy = s.v.Y[2] - s.v.Y[0];
   const bool front = s.fits ? ux * vy - vx * uy > 0 : (int64_t)ux * vy - (int64_t)vx * uy > 0;
   s.live = front && s.px1 >= s.px0 && s.py1 >= s.py0;
@@ -1305,72 +1316,192 @@ __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uin
 }
 
 // Any sub-triangle, 64-bit edge functions: samples first, first + step, .. of its box in
-// row order.  TEST: nothing is written; true when one of them has the pixel's final key.
+// row order, the edge functions stepped as in win_box.  TEST: nothing is written; true
+// when one of them has the pixel's final key.
 template <bool TEST>
 __device__ __forceinline__ bool win_rect64(const RasterArgs& A, const SV& a, const SV& b, const SV& c, uint32_t t, int px0,
                                            int py0, int px1, int py1, uint32_t first, uint32_t step) {
+  constexpr int N = 4;
+  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
+  if (first >= n) return false;
   const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
   const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
-  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
-  Put q;
-  for (uint32_t s = first; s < n; s += step) {
-    const int px = px0 + (int)(s % w), py = py0 + (int)(s / w);
-    const Edges E = edges_at(a, b, c, px, py);
-    const bool in = (E.e[0] > 0 || (E.e[0] == 0 && E.tl[0])) && (E.e[1] > 0 || (E.e[1] == 0 && E.tl[1])) &&
-                    (E.e[2] > 0 || (E.e[2] == 0 && E.tl[2]));
-    if (!in) continue;
-    float f = __fmul_rn(ll2float_rn(E.e[0]), a.zn);
-    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[1]), b.zn));
-    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[2]), c.zn));
-    const float d = __fmul_rn(f, invA);
-    if (!(d >= -1.0f && d <= 1.0f)) continue;
-    const uint32_t key = ordered(d), p = (uint32_t)py * (uint32_t)A.W + (uint32_t)px;
-    if (TEST) {
-      if (key <= zkey(A, p)) return true;
-    } else {
-      q.put(A, p, key, t);
-    }
-  }
-  if (!TEST) q.check(A, t);
-  return false;
-}
-
-// One queue record and its tiles for a large sub-triangle, at (entry e, first tile):
-// false when the queue or the tile table is full (the reserved record is then empty and
-// the reserved tiles have no owner).
-__device__ __forceinline__ bool win_queue(const RasterArgs& A, const int (&X)[3], const int (&Y)[3],
-                                          const float (&z)[3], int px0, int py0, int px1, int py1, bool fits,
-                                          uint32_t t, uint64_t e, uint64_t tile, uint32_t tiles) {
-  const bool ok = e < A.queue_cap && tile + tiles <= A.tile_cap;
-  if (e < A.queue_cap) {
-    BigTri bt;
+  const uint32_t sy = step / w, sx = step - sy * w, fy = first / w, fx = first - fy * w;
+  const Edges E = edges_at(a, b, c, px0 + (int)fx, py0 + (int)fy);
+  int64_t e[3], in_row[3], past[3];  // edge values; a step inside the row, one past its end
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      bt.X[i] = X[i];
-      bt.Y[i] = Y[i];
-      bt.zn[i] = z[i];
-    }
-    bt.px0 = ok ? px0 : 1;
-    bt.py0 = ok ? py0 : 1;
-    bt.px1 = ok ? px1 : 0;
-    bt.py1 = ok ? py1 : 0;
-    bt.tri = t;
-    bt.tile0 = (uint32_t)tile;
-    bt.pad = fits ? 1u : 0u;
-    A.queue[e] = bt;
+  for (int i = 0; i < 3; ++i) {
+    e[i] = E.e[i] - (E.tl[i] ? 0 : 1);  // (covered when none is negative)
+    in_row[i] = E.dy[i] * (int64_t)sy + E.dx[i] * (int64_t)sx;
+    past[i] = in_row[i] + E.dy[i] - E.dx[i] * (int64_t)w;
   }
-  for (uint64_t j = tile; j < tile + tiles && j < A.tile_cap; ++j) A.tile_owner[j] = ok ? (uint32_t)e : 0xFFFFFFFFu;
-  return ok;
+  const uint32_t ap = (uint32_t)A.W * sy + sx, bp = ap + (uint32_t)A.W - w;
+  uint32_t p = (uint32_t)(py0 + (int)fy) * (uint32_t)A.W + (uint32_t)px0 + fx, col = w - fx;  // col: pixels to the row's end
+  PutN<TEST ? 1 : N> later;
+  bool hit = false;
+  for (uint32_t s = first; s < n && !hit;) {
+    uint32_t key[N], pix[N];
+    bool on[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      pix[i] = p;
+      on[i] = s < n && (e[0] | e[1] | e[2]) >= 0;
+      key[i] = 0u;
+      if (on[i]) {
+        float f = __fmul_rn(ll2float_rn(e[0] + (E.tl[0] ? 0 : 1)), a.zn);
+        f = __fadd_rn(f, __fmul_rn(ll2float_rn(e[1] + (E.tl[1] ? 0 : 1)), b.zn));
+        f = __fadd_rn(f, __fmul_rn(ll2float_rn(e[2] + (E.tl[2] ? 0 : 1)), c.zn));
+        const float d = __fmul_rn(f, invA);
+        on[i] = d >= -1.0f && d <= 1.0f;
+        key[i] = ordered(d);
+      }
+      const bool wrap = col <= sx;
+      col = col - sx + (wrap ? w : 0u);
+      p += wrap ? bp : ap;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) e[k] += wrap ? past[k] : in_row[k];
+      s += step;
+    }
+    if constexpr (TEST) {
+      uint32_t z[N];
+#pragma unroll
+      for (int i = 0; i < N; ++i) z[i] = on[i] ? zkey(A, pix[i]) : 0u;
+#pragma unroll
+      for (int i = 0; i < N; ++i) hit |= on[i] && key[i] <= z[i];
+    } else {
+      later.put(A, t, on, key, pix);
+    }
+  }
+  if constexpr (!TEST) later.check(A, t);
+  return hit;
 }
 
-__device__ __forceinline__ uint32_t tiles_of(int w, int h) {
-  return (uint32_t)((w + kBigTile - 1) / kBigTile) * (uint32_t)((h + kBigTile - 1) / kBigTile);
+// Record e of the queue: a large sub-triangle whose tiles are numbered from `tile` on.
+// (Records and tiles are reserved by one atomic, so a later record has later tiles.)
+__device__ __forceinline__ void win_queue(const RasterArgs& A, const int (&X)[3], const int (&Y)[3],
+                                          const float (&z)[3], int px0, int py0, int px1, int py1, bool fits,
+                                          uint32_t t, uint32_t e, uint64_t tile) {
+  BigTri bt;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    bt.X[i] = X[i];
+    bt.Y[i] = Y[i];
+    bt.zn[i] = z[i];
+  }
+  bt.px0 = px0;
+  bt.py0 = py0;
+  bt.px1 = px1;
+  bt.py1 = py1;
+  bt.tri = t;
+  bt.tile0 = (uint32_t)tile;
+  bt.pad = (fits ? 0x80000000u : 0u) | (uint32_t)(tile >> 32);
+  A.queue[e] = bt;
+}
+
+__device__ __forceinline__ uint64_t first_tile(uint32_t tile0, uint32_t pad) {
+  return tile0 | (uint64_t)(pad & 0x7FFFFFFFu) << 32;
+}
+
+// Owners of each lane's record's tiles (none: tiles = 0) that the table has room for: few
+// by the lane itself, many by the whole warp (the exact pass of a 1080p view with two
+// clipped ground triangles: 361 us with every lane on its own, 22 so).  All lanes of the
+// warp call it.
+__device__ __forceinline__ void own_tiles(const RasterArgs& A, uint32_t e, uint64_t tile, uint32_t tiles) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t j0 = (uint32_t)(tile < A.tile_cap ? tile : A.tile_cap);
+  const uint32_t n = tiles < A.tile_cap - j0 ? tiles : A.tile_cap - j0;
+  if (n <= 8u)
+    for (uint32_t j = 0; j < n; ++j) A.tile_owner[j0 + j] = e;
+  for (uint32_t m = __ballot_sync(0xFFFFFFFFu, n > 8u); m; m &= m - 1u) {
+    const int src = __ffs(m) - 1;
+    const uint32_t we = __shfl_sync(0xFFFFFFFFu, e, src), wj = __shfl_sync(0xFFFFFFFFu, j0, src),
+                   wn = __shfl_sync(0xFFFFFFFFu, n, src);
+    for (uint32_t j = lane; j < wn; j += 32u) A.tile_owner[wj + j] = we;
+  }
+}
+
+// The record that tile g belongs to, the last one that starts at or before it: each round
+// the lanes look at 32 records evenly apart.
+__device__ __noinline__ uint32_t record_of(const RasterArgs& A, uint32_t n_ent, uint64_t g) {
+  const uint32_t lane = threadIdx.x & 31;
+  uint32_t lo = 0, hi = n_ent;
+  while (hi - lo > 1u) {
+    const uint32_t step = (hi - lo + 31u) / 32u, i = lo + lane * step;
+    bool before = false;
+    if (i < hi) {
+      const uint2 q = __ldcg(reinterpret_cast<const uint2*>(&A.queue[i].tile0));
+      before = first_tile(q.x, q.y) <= g;
+    }
+    lo += ((uint32_t)__popc(__ballot_sync(0xFFFFFFFFu, before)) - 1u) * step;  // (record lo starts at or before g)
+    hi = min(hi, lo + step);
+  }
+  return lo;
+}
+
+// Records of the queue and their tiles.  FULL: there may be more than the queue and the
+// owner table hold (tiles reserved past the last record belong to no one).
+struct Queued {
+  uint32_t records;
+  uint64_t tiles;
+};
+
+__device__ __forceinline__ bool overfull(const RasterArgs& A, unsigned long long st) {
+  return (st >> 40) > A.queue_cap || (st & ((1ull << 40) - 1)) > A.tile_cap;
+}
+
+template <bool FULL>
+__device__ __forceinline__ Queued queued(const RasterArgs& A, unsigned long long st) {
+  Queued n{(uint32_t)min(st >> 40, (unsigned long long)A.queue_cap), st & ((1ull << 40) - 1)};
+  if (FULL && (st >> 40) > A.queue_cap) {
+    const BigTri& q = A.queue[A.queue_cap - 1u];
+    n.tiles = first_tile(q.tile0, q.pad) + tiles_of(q.px1 - q.px0 + 1, q.py1 - q.py0 + 1);
+  }
+  return n;
+}
+
+// Tile::run(A, record, tile in it) for every tile of the queued records, a warp each.  The
+// table holds the owners of the first tile_cap tiles, four for each record there is room
+// for.  st: the queue's counter.  FULL: also the tiles past it (a few triangles that fill the view), in runs of
+// neighbours: the first one's record is looked up, the next ones' are the same or the next.
+// (Rasterized by the threads that set them up instead, 40 triangles that fill a 1080p
+// window take 1.7 s and 40 clipped ones 734 ms; so 0.69 and 0.33 ms.)
+template <class Tile, bool FULL>
+__device__ __forceinline__ void for_tiles(const RasterArgs& A, unsigned long long st, uint32_t bid, uint32_t nblk) {
+  const uint32_t warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = (nblk * blockDim.x) >> 5;
+  const Queued n = queued<FULL>(A, st);
+  if (n.records == 0u) return;
+  const uint32_t n_tab = FULL ? (uint32_t)min(n.tiles, (uint64_t)A.tile_cap) : (uint32_t)n.tiles;
+  for (uint32_t g = warp; g < n_tab; g += nwarps) {
+    const BigTri& q = A.queue[__ldcg(A.tile_owner + g)];
+    Tile::run(A, q, g - q.tile0);
+  }
+  if (!FULL) return;
+  const uint64_t rest = n.tiles - n_tab, each = (rest + nwarps - 1u) / nwarps;
+  const uint32_t run = each > 32u ? 32u : (uint32_t)each;
+  for (uint64_t i = (uint64_t)warp * run; i < rest; i += (uint64_t)nwarps * run) {
+    uint64_t g = n_tab + i;
+    uint32_t e = record_of(A, n.records, g);
+    for (uint32_t k = (uint32_t)min((uint64_t)run, rest - i); k; --k, ++g) {
+      uint64_t local = g - first_tile(A.queue[e].tile0, A.queue[e].pad);
+      if (local >= tiles_of(A.queue[e].px1 - A.queue[e].px0 + 1, A.queue[e].py1 - A.queue[e].py0 + 1)) {
+        ++e;
+        local = 0u;
+      }
+      Tile::run(A, A.queue[e], (uint32_t)local);
+    }
+  }
 }
 
 // A triangle that must be clipped (rare).  TEST as in win_rect64; else its sub-triangles
-// are rasterized here (small) or queued.
+// are rasterized here (small) or queued, their records first .. first + n - 1 returned
+// for their tiles' owners.
+struct Fan {
+  uint32_t first, n;
+};
+
 template <bool TEST>
-__device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4 c0, float4 c1, float4 c2) {
+__device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4 c0, float4 c1, float4 c2, Fan& fan) {
+  fan = Fan{0u, 0u};
   CV poly[kMaxPoly];
   poly[0] = CV{c0.x, c0.y, c0.z, c0.w};
   poly[1] = CV{c1.x, c1.y, c1.z, c1.w};
@@ -1384,23 +1515,43 @@ __device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4
   for (int i = 0; i < n; ++i)
     if (!(poly[i].w > 0.0f)) return false;
   SV sv[kMaxPoly];
+  uint32_t nq = 0;
+  uint64_t tiles = 0;
   for (int i = 0; i < n; ++i) sv[i] = project(poly[i], A.hx, A.hy);
+  if (!TEST) {
+    for (int i = 1; i + 1 < n; ++i) {
+      const Setup s = setup(sv[0], sv[i], sv[i + 1], A.W, A.H, false);
+      const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
+      if (s.A <= 0 || w <= 0 || h <= 0 || w * h <= kSmallMaxPix) continue;
+      ++nq;
+      tiles += tiles_of(w, h);
+    }
+  }
+  uint64_t e = 0, tile = 0;
+  if (nq) {
+    const unsigned long long old = atomicAdd(&A.ctr->big, ((unsigned long long)nq << 40) | (unsigned long long)tiles);
+    e = old >> 40;
+    tile = old & ((1ull << 40) - 1);
+    if (e < A.queue_cap) fan = Fan{(uint32_t)e, min(nq, A.queue_cap - (uint32_t)e)};
+  }
   for (int i = 1; i + 1 < n; ++i) {
     const SV &a = sv[0], &b = sv[i], &c = sv[i + 1];
     const Setup s = setup(a, b, c, A.W, A.H, false);
-    if (s.A <= 0 || s.px1 < s.px0 || s.py1 < s.py0) continue;
+    const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
+    if (s.A <= 0 || w <= 0 || h <= 0) continue;
     if (TEST) {
       if (win_rect64<true>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u)) return true;
       continue;
     }
-    const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
     if (w * h > kSmallMaxPix) {
-      const uint32_t tiles = tiles_of(w, h);
-      const unsigned long long old = atomicAdd(&A.ctr->big, (1ull << 40) | (unsigned long long)tiles);
-      const int X[3] = {(int)a.X, (int)b.X, (int)c.X}, Y[3] = {(int)a.Y, (int)b.Y, (int)c.Y};
-      const float z[3] = {a.zn, b.zn, c.zn};
-      if (win_queue(A, X, Y, z, s.px0, s.py0, s.px1, s.py1, false, t, old >> 40, old & ((1ull << 40) - 1), tiles))
+      if (e < A.queue_cap) {
+        const int X[3] = {(int)a.X, (int)b.X, (int)c.X}, Y[3] = {(int)a.Y, (int)b.Y, (int)c.Y};
+        const float z[3] = {a.zn, b.zn, c.zn};
+        win_queue(A, X, Y, z, s.px0, s.py0, s.px1, s.py1, false, t, (uint32_t)e, tile);
+        ++e;
+        tile += tiles_of(w, h);
         continue;
+      }
     }
     win_rect64<false>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u);
   }
@@ -1447,25 +1598,8 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
         if (kind == 2) tiles = tiles_of(w, h);
       }
     }
-    const uint32_t mids = __ballot_sync(0xFFFFFFFFu, kind == 3);
-    if (mids) {
-      uint32_t o = 0;
-      if (lane == 0) o = atomicAdd(&A.ctr->n_mid[list][0], (uint32_t)__popc(mids));
-      o = __shfl_sync(0xFFFFFFFFu, o, 0) + __popc(mids & ((1u << lane) - 1u));
-      if (kind == 3) {
-        if (o < lcap) {
-          float4* d = reinterpret_cast<float4*>(A.cand + lbase + o);
-          d[0] = make_float4(__int_as_float(E.v.X[0]), __int_as_float(E.v.Y[0]), __int_as_float(E.v.X[1]),
-                             __int_as_float(E.v.Y[1]));
-          d[1] = make_float4(__int_as_float(E.v.X[2]), __int_as_float(E.v.Y[2]),
-                             __int_as_float(E.px0 | (E.py0 << 16)), __int_as_float(E.px1 | (E.py1 << 16)));
-          d[2] = make_float4(E.v.z[0], E.v.z[1], E.v.z[2], __uint_as_float(t));
-        } else {
-          win_box<4>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
-        }
-      }
-    }
-    // large triangles of the warp reserve queue records and tiles with one atomic
+    // large triangles of the warp reserve queue records and tiles with one atomic; a
+    // triangle that finds no record any more is listed as a mid-size one, whatever its size
     const uint32_t bigs = __ballot_sync(0xFFFFFFFFu, kind == 2);
     if (bigs) {
       uint32_t tpre = tiles;  // inclusive prefix of tiles over the warp
@@ -1479,11 +1613,33 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
       if (lane == 0)
         old = atomicAdd(&A.ctr->big, ((unsigned long long)__popc(bigs) << 40) | (unsigned long long)ttot);
       old = __shfl_sync(0xFFFFFFFFu, old, 0);
-      if (kind == 2 &&
-          !win_queue(A, E.v.X, E.v.Y, E.v.z, E.px0, E.py0, E.px1, E.py1, E.fits, t,
-                     (old >> 40) + __popc(bigs & ((1u << lane) - 1u)), (old & ((1ull << 40) - 1)) + (tpre - tiles), tiles)) {
-        const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
-        win_rect64<false>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
+      const uint64_t e = (old >> 40) + __popc(bigs & ((1u << lane) - 1u));
+      const uint64_t tile = (old & ((1ull << 40) - 1)) + (tpre - tiles);
+      if (kind == 2 && e < A.queue_cap) {
+        win_queue(A, E.v.X, E.v.Y, E.v.z, E.px0, E.py0, E.px1, E.py1, E.fits, t, (uint32_t)e, tile);
+      } else {
+        tiles = 0;
+        if (kind == 2) kind = 3;
+      }
+      own_tiles(A, (uint32_t)e, tile, tiles);
+    }
+    const uint32_t mids = __ballot_sync(0xFFFFFFFFu, kind == 3);
+    if (mids) {
+      uint32_t o = 0;
+      if (lane == 0) o = atomicAdd(&A.ctr->n_mid[list][0], (uint32_t)__popc(mids));
+      o = __shfl_sync(0xFFFFFFFFu, o, 0) + __popc(mids & ((1u << lane) - 1u));
+      if (kind == 3) {
+        if (o < lcap) {  // (always: the list has room for every survivor its blocks see)
+          float4* d = reinterpret_cast<float4*>(A.cand + lbase + o);
+          d[0] = make_float4(__int_as_float(E.v.X[0]), __int_as_float(E.v.Y[0]), __int_as_float(E.v.X[1]),
+                             __int_as_float(E.v.Y[1]));
+          d[1] = make_float4(__int_as_float(E.v.X[2]), __int_as_float(E.v.Y[2]),
+                             __int_as_float(E.px0 | (E.py0 << 16)),
+                             __int_as_float(E.px1 | (E.py1 << 16) | (E.fits ? 0 : (int)0x80000000)));
+          d[2] = make_float4(E.v.z[0], E.v.z[1], E.v.z[2], __uint_as_float(t));
+        } else {
+          set_status(A.ctr, FA_E_CAPACITY);
+        }
       }
     }
     if (!grouped) {
@@ -1508,51 +1664,53 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
   // then the (rare) triangles that need clipping, from the front blocks' regions
   if (!__syncthreads_or(clipped != 0u)) return;  // (and pre is reused)
   const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
-  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
-    const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
-    const uint32_t* f = A.idx + 3 * (size_t)t;
-    const Mat4 M = DEV_M ? load_mat(A.Mdev) : A.M;
-    win_clipped<false>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
-                       load_clip(M, A.pos, __ldg(f + 2)));
+  for (uint32_t base = bid * blockDim.x + (threadIdx.x & ~31u); base < nc; base += stride) {
+    const uint32_t i = base + lane;
+    Fan fan{0u, 0u};
+    if (i < nc) {
+      const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
+      const uint32_t* f = A.idx + 3 * (size_t)t;
+      const Mat4 M = DEV_M ? load_mat(A.Mdev) : A.M;
+      win_clipped<false>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
+                         load_clip(M, A.pos, __ldg(f + 2)), fan);
+    }
+    // a record of each lane's fan after the other
+    for (uint32_t q = 0; __any_sync(0xFFFFFFFFu, q < fan.n); ++q) {
+      uint32_t tiles = 0;
+      uint64_t tile = 0;
+      if (q < fan.n) {
+        const BigTri& r = A.queue[fan.first + q];
+        tile = first_tile(r.tile0, r.pad);
+        tiles = tiles_of(r.px1 - r.px0 + 1, r.py1 - r.py0 + 1);
+      }
+      own_tiles(A, fan.first + q, tile, tiles);
+    }
   }
 }
 
-// The queued tiles, a warp each, then the mid-size lists.
-__device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
-  __shared__ uint32_t pre[kMidLists + 1];
-  const uint32_t lane = threadIdx.x & 31;
-  __syncthreads();  // pre of an earlier item of the same block is free
-  const unsigned long long st = __ldcg(&A.ctr->big);
-  if (threadIdx.x < 32) {
-    uint32_t c = 0;
-    if (lane < A.mid_lists) c = min(__ldcg(&A.ctr->n_mid[lane][0]), mid_base(A, lane + 1u) - mid_base(A, lane));
-    uint32_t x = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
-      if (lane >= (unsigned)o) x += y;
-    }
-    pre[lane + 1] = x;
-    if (lane == 0) pre[0] = 0u;
+// The listed record of position i, pre: where each list starts.
+__device__ __forceinline__ const float4* mid_record(const RasterArgs& A, const uint32_t* pre, uint32_t i) {
+  uint32_t lo = 0, hi = kMidLists;  // pre[lo] <= i < pre[hi]
+  while (hi - lo > 1u) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if (pre[mid] <= i) lo = mid;
+    else hi = mid;
   }
-  const uint32_t warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = (nblk * blockDim.x) >> 5;
-  const uint32_t n_ent = (uint32_t)min((unsigned long long)A.queue_cap, st >> 40);
-  const uint32_t n_tiles = n_ent ? (uint32_t)min((unsigned long long)A.tile_cap, st & ((1ull << 40) - 1)) : 0u;
-  for (uint32_t g = warp; g < n_tiles; g += nwarps) {
-    const uint32_t lo = __ldcg(A.tile_owner + g);
-    if (lo >= n_ent) continue;
-    const BigTri& q = A.queue[lo];
-    const int px0 = q.px0, py0 = q.py0, px1 = q.px1, py1 = q.py1;
-    if (px1 < px0 || py1 < py0) continue;
-    const uint32_t tx_n = (uint32_t)((px1 - px0 + kBigTile) / kBigTile);
-    const uint32_t local = g - q.tile0;
-    const int bx = px0 + (int)(local % tx_n) * kBigTile, by = py0 + (int)(local / tx_n) * kBigTile;
-    if (by > py1) continue;
+  return reinterpret_cast<const float4*>(A.cand + mid_base(A, lo) + (i - pre[lo]));
+}
+
+// One 16x16 tile of a queued record, by a warp.
+struct PutTile {
+  static __device__ __forceinline__ void run(const RasterArgs& A, const BigTri& q, uint32_t local) {
+    const uint32_t lane = threadIdx.x & 31;
+    const int px1 = q.px1, py1 = q.py1;
+    const uint32_t tx_n = (uint32_t)((px1 - q.px0 + kBigTile) / kBigTile);
+    const int bx = q.px0 + (int)(local % tx_n) * kBigTile, by = q.py0 + (int)(local / tx_n) * kBigTile;
     const uint32_t t = q.tri;
     const int px = bx + (int)(lane % kBigTile), py_first = by + (int)(lane / kBigTile);
     const int py_last = min(by + kBigTile - 1, py1);
     Put put;
-    if (q.pad) {
+    if (q.pad >> 31) {
       const Tri32 v{{q.X[0], q.X[1], q.X[2]}, {q.Y[0], q.Y[1], q.Y[2]}, {q.zn[0], q.zn[1], q.zn[2]}};
       const Edges32 E = edges32(v, px, py_first);
       int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2];
@@ -1600,27 +1758,77 @@ __device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid
     }
     put.check(A, t);
   }
+};
+
+// The listed sub-triangles that found no queue record and are too large for 32 bits, a
+// warp each (rare).
+__device__ __forceinline__ void mid_wide(const RasterArgs& A, uint32_t bid, uint32_t nblk, const uint32_t* pre) {
+  const uint32_t n = pre[kMidLists], lane = threadIdx.x & 31;
+  for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> 5; i < n; i += (nblk * blockDim.x) >> 5) {
+    const float4* s = mid_record(A, pre, i);
+    const float4 f0 = __ldcg(s), f1 = __ldcg(s + 1), f2 = __ldcg(s + 2);
+    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
+    if ((int)b1 >= 0) continue;
+    const SV a{__float_as_int(f0.x), __float_as_int(f0.y), f2.x}, b{__float_as_int(f0.z), __float_as_int(f0.w), f2.y},
+        c{__float_as_int(f1.x), __float_as_int(f1.y), f2.z};
+    win_rect64<false>(A, a, b, c, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu),
+                      (int)((b1 >> 16) & 0x7FFFu), lane, 32u);
+  }
+}
+
+// Where each mid-size list starts, pre[0] .. pre[kMidLists] (seen after a barrier).
+__device__ __forceinline__ void mid_prefix(const RasterArgs& A, uint32_t* pre) {
+  const uint32_t lane = threadIdx.x & 31;
+  __syncthreads();  // pre of an earlier item of the same block is free
+  if (threadIdx.x < 32) {
+    uint32_t c = 0;
+    if (lane < A.mid_lists) c = min(__ldcg(&A.ctr->n_mid[lane][0]), mid_base(A, lane + 1u) - mid_base(A, lane));
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+      if (lane >= (unsigned)o) x += y;
+    }
+    pre[lane + 1] = x;
+    if (lane == 0) pre[0] = 0u;
+  }
+}
+
+// The queued tiles, a warp each, then the mid-size lists.
+template <bool FULL>
+__device__ __forceinline__ void depth_win(const RasterArgs& A, unsigned long long st, uint32_t bid, uint32_t nblk,
+                                          uint32_t* pre) {
+  for_tiles<PutTile, FULL>(A, st, bid, nblk);
   __syncthreads();
   const uint32_t n = pre[kMidLists], stride = nblk * blockDim.x;
   uint32_t lg = kMinLanes;
   while (lg < 5u && ((uint64_t)n << (lg + 1u)) <= stride) ++lg;
   const uint32_t sub = threadIdx.x & ((1u << lg) - 1u);
   for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> lg; i < n; i += stride >> lg) {
-    uint32_t lo = 0, hi = kMidLists;  // pre[lo] <= i < pre[hi]
-    while (hi - lo > 1u) {
-      const uint32_t mid = (lo + hi) >> 1;
-      if (pre[mid] <= i) lo = mid;
-      else hi = mid;
-    }
-    const float4* s = reinterpret_cast<const float4*>(A.cand + mid_base(A, lo) + (i - pre[lo]));
+    const float4* s = mid_record(A, pre, i);
     const float4 f0 = __ldcs(s), f1 = __ldcs(s + 1), f2 = __ldcs(s + 2);
     const Tri32 v{{__float_as_int(f0.x), __float_as_int(f0.z), __float_as_int(f1.x)},
                   {__float_as_int(f0.y), __float_as_int(f0.w), __float_as_int(f1.y)},
                   {f2.x, f2.y, f2.z}};
-    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
-    win_box<4, true>(A, v, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu), (int)(b1 >> 16),
-               (int)sub, 1 << lg);
+    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w), t = __float_as_uint(f2.w);
+    const int px0 = (int)(b0 & 0xFFFFu), py0 = (int)(b0 >> 16), px1 = (int)(b1 & 0xFFFFu), py1 = (int)(b1 >> 16);
+    if ((int)b1 >= 0) win_box<4, true>(A, v, t, px0, py0, px1, py1, (int)sub, 1 << lg);
   }
+  if (FULL) mid_wide(A, bid, nblk, pre);
+}
+
+__device__ __noinline__ void depth_win_full(const RasterArgs& A, uint32_t bid, uint32_t nblk, uint32_t* pre) {
+  depth_win<true>(A, __ldcg(&A.ctr->big), bid, nblk, pre);
+}
+
+// (the full form on its own: in one body with the other it takes that one's registers,
+// and 60 patches at 1080p, which have no large triangle, 57 us instead of 39)
+__device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  __shared__ uint32_t pre[kMidLists + 1];
+  const unsigned long long st = __ldcg(&A.ctr->big);
+  mid_prefix(A, pre);
+  if (overfull(A, st)) depth_win_full(A, bid, nblk, pre);
+  else depth_win<false>(A, st, bid, nblk, pre);
 }
 
 // Sets triangle t's visible bit.
@@ -1674,8 +1882,9 @@ __device__ __noinline__ void mark_all(const RasterArgs& A, uint32_t bid, uint32_
   for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
     const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
     const uint32_t* f = A.idx + 3 * (size_t)t;
+    Fan fan;
     if (win_clipped<true>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
-                          load_clip(M, A.pos, __ldg(f + 2))))
+                          load_clip(M, A.pos, __ldg(f + 2)), fan))
       win_mark(A, t);
   }
 }
