@@ -1162,7 +1162,11 @@ __device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4&
   return s;
 }
 
+// (Once there are more ties than the list holds their number does not matter: it is no
+// longer added to, so that it cannot wrap, however many samples of a view are equal.  It
+// stays below tie_cap + the threads of the grid.)
 __device__ __forceinline__ void note_tie(const RasterArgs& A, uint32_t pix, uint32_t key, uint32_t t0, uint32_t t1) {
+  if (__ldcg(&A.ctr->n_ties) > A.tie_cap) return;
   const uint32_t i = atomicAdd(&A.ctr->n_ties, 1u);
   if (i < A.tie_cap) A.ties[i] = make_uint4(pix, key, t0, t1);
 }
