@@ -191,7 +191,8 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
     ctx->xedge = static_cast<uint2*>(ctx->surv_clip);
     ctx->vis = ctx->xedge + nblocks * 3072;
     ctx->ties = reinterpret_cast<uint4*>(pk.rec8);
-    ctx->tie_cap = (uint32_t)((uint64_t)kMaxScales * pk.max_chunks * kChunk / 2);
+    static_assert(kTies * sizeof(uint4) <= (uint64_t)kMaxScales * kChunk * sizeof(uint2),
+                  "the ties fit the push records of one chunk");
   }
   pk.ctr = ctx->ctr;
   pk.count = nullptr;

@@ -37,6 +37,7 @@ constexpr uint32_t kDefaultPushThreads = 512;  // threads of a candidate's push 
 constexpr uint32_t kPschedWords = 64;          // schedule state of a single-view persistent launch
 
 constexpr int kMidLists = 32;  // lists of mid-size sub-triangles (one counter each, so that few warps share one)
+constexpr uint32_t kTies = 1u << 17;  // listed pixels where two triangles have the same depth key
 
 struct DevCounters {
   int32_t status;          // sticky fa_status of the context
@@ -120,8 +121,7 @@ struct fa_ctx {
   void* arena;
   fa::DevCounters* ctr;
   uint32_t* zbuf;        // [max_w * max_h] depth keys, or 64-bit key | triangle
-  uint4* ties;           // [tie_cap] pixels where two triangles have the same key (in pack.rec8)
-  uint32_t tie_cap;
+  uint4* ties;           // [kTies] pixels where two triangles have the same key (in pack.rec8)
   uint32_t* zmax;        // [ceil(max_w / 16) * ceil(max_h / 16)] largest depth key per 16x16 tile
   uint32_t* tile_flag;   // [ceil(max_tris / 1024)] tile has a visible triangle (this frame)
   uint32_t* tile_list;   // [ceil(max_tris / 1024)] those tiles, in the order the marking found them

@@ -85,8 +85,9 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
   }
   mark(ctx, "k_raster_mark", s);
   // one wave of four resident blocks per SM: each block scans the region counts once
-  if (A.win)  // (blocks of 64 x 32 pixels)
-    launch_k(k_raster_mark<kMarkWinners>, std::min(((W + 63) / 64) * ((H + 31) / 32), 152u * 8u), 256, 0, s, A);
+  if (A.win)  // (blocks of 64 x 32 pixels; enough threads for many triangles in a small window, should ties overflow)
+    launch_k(k_raster_mark<kMarkWinners>,
+             std::min(std::max(((W + 63) / 64) * ((H + 31) / 32), (mesh->T + 255) / 256), 152u * 8u), 256, 0, s, A);
   else
     launch_k(cons ? k_raster_mark<kMarkConservative> : k_raster_mark<kMarkSamples>, 152 * 4, 256, 0, s, A);
   if (A.win && cons) {

@@ -339,8 +339,7 @@ struct RasterArgs {
   // single-pass visibility (see "winners" below): the depth buffer holds key << 32 | triangle
   int win;
   unsigned long long* zid;  // [W * H], the same memory as zbuf
-  uint4* ties;              // [tie_cap] (pixel, key, triangle, triangle) of equal keys
-  uint32_t tie_cap;
+  uint4* ties;              // [kTies] (pixel, key, triangle, triangle) of equal keys
   uint32_t mid_blocks, mid_lists, mid_per_block;  // exact pass's blocks, mid-size lists, slots per block
 };
 
@@ -937,6 +936,55 @@ __device__ __forceinline__ void note_tile(const RasterArgs& A, uint32_t tile) {
     A.tile_list[atomicAdd(&A.ctr->n_vtiles, 1u)] = tile;
 }
 
+// The depth key of a pixel: the buffer's word, or the upper half of key << 32 | triangle.
+template <bool WIN>
+__device__ __forceinline__ uint32_t* zword(const RasterArgs& A, size_t pix) {
+  return WIN ? reinterpret_cast<uint32_t*>(A.zid) + 2 * pix + 1 : A.zbuf + pix;
+}
+
+// One 16x16 tile of a queued record, by a warp, PASS as in sample().
+template <int PASS, bool WIN>
+__device__ __forceinline__ void raster_tile(const RasterArgs& A, const BigTri& q, uint32_t local) {
+  const uint32_t lane = threadIdx.x & 31;
+  const int px0 = q.px0, py0 = q.py0, px1 = q.px1, py1 = q.py1;
+  // marking: another tile of the sub-triangle may have marked its triangle already
+  // (one answer for the warp, which stays together below)
+  if (PASS >= 1 && __any_sync(0xFFFFFFFFu, (__ldcg(A.vt + (q.tri >> 5)) >> (q.tri & 31)) & 1u)) return;
+  const uint32_t tx_n = (uint32_t)((px1 - px0 + kBigTile) / kBigTile);
+  const int bx = px0 + (int)(local % tx_n) * kBigTile, by = py0 + (int)(local / tx_n) * kBigTile;
+  if (PASS >= 1 && !WIN && hidden_by_tiles(A, q.zn[0], q.zn[1], q.zn[2], bx, by, min(bx + kBigTile - 1, px1),
+                                   min(by + kBigTile - 1, py1)))
+    return;
+  SV a{q.X[0], q.Y[0], q.zn[0]}, b{q.X[1], q.Y[1], q.zn[1]}, c{q.X[2], q.Y[2], q.zn[2]};
+  const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
+  const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
+  const float zmin = fminf(a.zn, fminf(b.zn, c.zn)), zmax = fmaxf(a.zn, fmaxf(b.zn, c.zn));
+  bool vis = false;
+  const int px = bx + (int)(lane % kBigTile), py_first = by + (int)(lane / kBigTile);
+  const Edges E = edges_at(a, b, c, px, py_first);
+  int64_t e[3] = {E.e[0], E.e[1], E.e[2]};
+  // only the tile's rows inside the box (the last tile row of a box is often
+  // short); the same trip count in every lane
+  const int rows = min(by + kBigTile - 1, py1) - by + 1;
+  const int steps = (rows + 32 / kBigTile - 1) / (32 / kBigTile);
+#pragma unroll 1
+  for (int k = 0; k < steps; ++k) {
+    const int py = py_first + k * (32 / kBigTile);
+    if (px <= px1 && py <= py1)
+      vis |= sample<PASS>(E, e, a, b, c, invA, zword<WIN>(A, (size_t)py * A.W + px), zmin, zmax);
+    if (PASS >= 1 && __any_sync(0xFFFFFFFFu, vis)) break;
+    e[0] += E.dy[0] * (32 / kBigTile);
+    e[1] += E.dy[1] * (32 / kBigTile);
+    e[2] += E.dy[2] * (32 / kBigTile);
+  }
+  if (PASS >= 1) {
+    if (__any_sync(0xFFFFFFFFu, vis) && lane == 0) {
+      atomicOr(A.vt + (q.tri >> 5), 1u << (q.tri & 31));
+      note_tile(A, q.tri >> 10);
+    }
+  }
+}
+
 // Large sub-triangles: one warp per 16x16 tile of a queued record (grid-stride).
 template <int PASS>
 __device__ __forceinline__ void big_tiles(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
@@ -958,40 +1006,7 @@ __device__ __forceinline__ void big_tiles(const RasterArgs& A, uint32_t bid, uin
     const uint32_t ty_n = (uint32_t)((py1 - py0 + kBigTile) / kBigTile);
     const uint64_t local = g - q.tile0;
     if (local >= (uint64_t)tx_n * ty_n) continue;
-    // marking: another tile of the sub-triangle may have marked its triangle already
-    if (PASS >= 1 && ((__ldcg(A.vt + (q.tri >> 5)) >> (q.tri & 31)) & 1u)) continue;
-    const int bx = px0 + (int)(local % tx_n) * kBigTile, by = py0 + (int)(local / tx_n) * kBigTile;
-    if (PASS >= 1 && hidden_by_tiles(A, q.zn[0], q.zn[1], q.zn[2], bx, by, min(bx + kBigTile - 1, px1),
-                                     min(by + kBigTile - 1, py1)))
-      continue;
-    SV a{q.X[0], q.Y[0], q.zn[0]}, b{q.X[1], q.Y[1], q.zn[1]}, c{q.X[2], q.Y[2], q.zn[2]};
-    const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
-    const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
-    const float zmin = fminf(a.zn, fminf(b.zn, c.zn)), zmax = fmaxf(a.zn, fmaxf(b.zn, c.zn));
-    bool vis = false;
-    const int px = bx + (int)(lane % kBigTile), py_first = by + (int)(lane / kBigTile);
-    const Edges E = edges_at(a, b, c, px, py_first);
-    int64_t e[3] = {E.e[0], E.e[1], E.e[2]};
-    // only the tile's rows inside the box (the last tile row of a box is often
-    // short); the same trip count in every lane
-    const int rows = min(by + kBigTile - 1, py1) - by + 1;
-    const int steps = (rows + 32 / kBigTile - 1) / (32 / kBigTile);
-#pragma unroll 1
-    for (int k = 0; k < steps; ++k) {
-      const int py = py_first + k * (32 / kBigTile);
-      if (px <= px1 && py <= py1)
-        vis |= sample<PASS>(E, e, a, b, c, invA, A.zbuf + (size_t)py * A.W + px, zmin, zmax);
-      if (PASS >= 1 && __any_sync(0xFFFFFFFFu, vis)) break;
-      e[0] += E.dy[0] * (32 / kBigTile);
-      e[1] += E.dy[1] * (32 / kBigTile);
-      e[2] += E.dy[2] * (32 / kBigTile);
-    }
-    if (PASS >= 1) {
-      if (__any_sync(0xFFFFFFFFu, vis) && lane == 0) {
-        atomicOr(A.vt + (q.tri >> 5), 1u << (q.tri & 31));
-        note_tile(A, q.tri >> 10);
-      }
-    }
+    raster_tile<PASS, false>(A, q, (uint32_t)local);
   }
 }
 
@@ -1084,8 +1099,8 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
 // rasterization.  Two triangles with the same key at a pixel are told by the returned
 // old value: the key a pixel ends with stays there once it has arrived, so every later
 // triangle with that key sees it and lists the pair; the marking pass marks the pairs
-// whose key is still the pixel's.  If the list overflows, the marking pass tests every
-// survivor against the buffer instead (mark_all).
+// whose key is still the pixel's.  If the list overflows (coincident geometry), the marking
+// pass tests what is not marked against the buffer instead (mark_all).
 //
 // Three sizes of sub-triangles, so that the lanes of a warp have like work: boxes of at
 // most kSmallMaxPix pixels are rasterized where they are set up (exact pass); boxes of
@@ -1109,6 +1124,7 @@ __device__ __forceinline__ void depth_big_body(const RasterArgs& A, uint32_t bid
 // us, 60 patches at 1080p 247 -> 83, 200 icospheres at 1080p 107 -> 62, one patch of
 // 7,938 triangles at 1080p 52 -> 40 (events around each kernel, GB300).
 constexpr int kMidPix = 256;  // (512: the same)
+constexpr uint32_t kMarkBlocks = 152u * 4u;  // resident blocks of the marking kernel
 constexpr uint32_t kMinLanes = 2;  // log2 of the fewest lanes a mid-size box gets
 constexpr int kSpan32 = 96 * kSub;  // side of a sub-triangle with 32-bit edge functions
 
@@ -1162,13 +1178,24 @@ __device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4&
   return s;
 }
 
-// (Once there are more ties than the list holds their number does not matter: it is no
-// longer added to, so that it cannot wrap, however many samples of a view are equal.  It
-// stays below tie_cap + the threads of the grid.)
+// Set once this block has found the tie list full (cleared before a pass's first sample).
+__device__ __forceinline__ volatile uint32_t* ties_full() {
+  __shared__ uint32_t full;
+  return &full;
+}
+
+// Lists a tie.  A block that has found the list full adds no more: the number of ties does
+// not matter then, a count that stays below the list's room plus the threads of the grid
+// cannot wrap however many samples of a view are equal, and the counter's atomics, all on
+// one word, do not hold the samples up (depth pass of eight copies of a patch 303 -> 74
+// us).  (The mid-size boxes' loop is sensitive to this function's form: 330 us on a
+// 3.2M-triangle floor; with lists by SM and by block, with the flag kept from the compiler
+// no longer, with the counter read instead of the flag, 340 to 500.)
 __device__ __forceinline__ void note_tie(const RasterArgs& A, uint32_t pix, uint32_t key, uint32_t t0, uint32_t t1) {
-  if (__ldcg(&A.ctr->n_ties) > A.tie_cap) return;
+  if (*ties_full()) return;
   const uint32_t i = atomicAdd(&A.ctr->n_ties, 1u);
-  if (i < A.tie_cap) A.ties[i] = make_uint4(pix, key, t0, t1);
+  if (i < kTies) A.ties[i] = make_uint4(pix, key, t0, t1);
+  else *ties_full() = 1u;
 }
 
 // The samples a thread has put: the returned value of one is looked at when the next
@@ -1238,6 +1265,10 @@ __device__ __forceinline__ void put_n(const RasterArgs& A, uint32_t t, const boo
     old[i] = ~0ull;
     if (on[i]) old[i] = atomicMin(A.zid + pix[i], ((unsigned long long)key[i] << 32) | t);
   }
+  bool any = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) any |= on[i] && (uint32_t)(old[i] >> 32) == key[i];
+  if (!any) return;
 #pragma unroll
   for (int i = 0; i < N; ++i)
     if (on[i] && (uint32_t)(old[i] >> 32) == key[i] && (uint32_t)old[i] != t)
@@ -1280,13 +1311,31 @@ struct PutN {
   }
 };
 
+// One of a thread's N samples (those that are on) has the pixel's final key.
+template <int N>
+__device__ __forceinline__ bool test_n(const RasterArgs& A, const bool (&on)[N], const uint32_t (&key)[N],
+                                       const uint32_t (&pix)[N]) {
+  uint32_t z[N];
+  bool hit = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) z[i] = on[i] ? zkey(A, pix[i]) : 0u;
+#pragma unroll
+  for (int i = 0; i < N; ++i) hit |= on[i] && key[i] <= z[i];
+  return hit;
+}
+
+// What becomes of the samples: put at once, put with the returned values looked at later,
+// or (nothing is written) tested against the final keys.
+enum Samples { kPut, kPutLater, kTest };
+
 // Samples first, first + step, .. (row order) of a 32-bit sub-triangle's box, N at a time
-// so that their atomics overlap.  step lanes side by side then put neighbouring pixels.
-template <int N, bool LATER = false>
-__device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uint32_t t, int px0, int py0, int px1,
+// so that their atomics or loads overlap.  step lanes side by side then take neighbouring
+// pixels.  kTest: true when one of them has the pixel's final key.
+template <int N, Samples DO>
+__device__ __forceinline__ bool win_box(const RasterArgs& A, const Tri32& v, uint32_t t, int px0, int py0, int px1,
                                         int py1, int first, int step) {
   const int w = px1 - px0 + 1, n = w * (py1 - py0 + 1);
-  if (first >= n) return;
+  if (first >= n) return false;
   const int sy = step == 1 ? (w == 1 ? 1 : 0) : step / w, sx = step - sy * w;  // step = sy rows and sx < w pixels
   const int fy = first / w, fx = first - fy * w;
   const Edges32 E = edges32(v, px0 + fx, py0 + fy);
@@ -1296,7 +1345,7 @@ __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uin
   const uint32_t ap = (uint32_t)(A.W * sy + sx), bp = ap + (uint32_t)(A.W - w);
   int e0 = E.e[0], e1 = E.e[1], e2 = E.e[2], col = w - fx;  // col: pixels to the row's end
   uint32_t p = (uint32_t)(py0 + fy) * (uint32_t)A.W + (uint32_t)(px0 + fx);
-  PutN<LATER ? N : 1> later;
+  PutN<DO == kPutLater ? N : 1> later;
   for (int left = n - 1 - first; left >= 0;) {  // (negative once the box is done)
     uint32_t key[N], pix[N];
     bool on[N];
@@ -1313,71 +1362,43 @@ __device__ __forceinline__ void win_box(const RasterArgs& A, const Tri32& v, uin
       p += wrap ? bp : ap;
       left -= step;
     }
-    if constexpr (LATER) later.put(A, t, on, key, pix);
-    else put_n(A, t, on, key, pix);
+    if constexpr (DO == kPutLater) later.put(A, t, on, key, pix);
+    else if constexpr (DO == kPut) put_n(A, t, on, key, pix);
+    else if (test_n(A, on, key, pix)) return true;
   }
-  if constexpr (LATER) later.check(A, t);
+  if constexpr (DO == kPutLater) later.check(A, t);
+  return false;
 }
 
 // Any sub-triangle, 64-bit edge functions: samples first, first + step, .. of its box in
-// row order, the edge functions stepped as in win_box.  TEST: nothing is written; true
-// when one of them has the pixel's final key.
+// row order.  TEST: nothing is written; true when one of them has the pixel's final key.
 template <bool TEST>
 __device__ __forceinline__ bool win_rect64(const RasterArgs& A, const SV& a, const SV& b, const SV& c, uint32_t t, int px0,
                                            int py0, int px1, int py1, uint32_t first, uint32_t step) {
-  constexpr int N = 4;
-  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
-  if (first >= n) return false;
   const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
   const float invA = __fdiv_rn(1.0f, ll2float_rn(Ar));
-  const uint32_t sy = step / w, sx = step - sy * w, fy = first / w, fx = first - fy * w;
-  const Edges E = edges_at(a, b, c, px0 + (int)fx, py0 + (int)fy);
-  int64_t e[3], in_row[3], past[3];  // edge values; a step inside the row, one past its end
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    e[i] = E.e[i] - (E.tl[i] ? 0 : 1);  // (covered when none is negative)
-    in_row[i] = E.dy[i] * (int64_t)sy + E.dx[i] * (int64_t)sx;
-    past[i] = in_row[i] + E.dy[i] - E.dx[i] * (int64_t)w;
-  }
-  const uint32_t ap = (uint32_t)A.W * sy + sx, bp = ap + (uint32_t)A.W - w;
-  uint32_t p = (uint32_t)(py0 + (int)fy) * (uint32_t)A.W + (uint32_t)px0 + fx, col = w - fx;  // col: pixels to the row's end
-  PutN<TEST ? 1 : N> later;
-  bool hit = false;
-  for (uint32_t s = first; s < n && !hit;) {
-    uint32_t key[N], pix[N];
-    bool on[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      pix[i] = p;
-      on[i] = s < n && (e[0] | e[1] | e[2]) >= 0;
-      key[i] = 0u;
-      if (on[i]) {
-        float f = __fmul_rn(ll2float_rn(e[0] + (E.tl[0] ? 0 : 1)), a.zn);
-        f = __fadd_rn(f, __fmul_rn(ll2float_rn(e[1] + (E.tl[1] ? 0 : 1)), b.zn));
-        f = __fadd_rn(f, __fmul_rn(ll2float_rn(e[2] + (E.tl[2] ? 0 : 1)), c.zn));
-        const float d = __fmul_rn(f, invA);
-        on[i] = d >= -1.0f && d <= 1.0f;
-        key[i] = ordered(d);
-      }
-      const bool wrap = col <= sx;
-      col = col - sx + (wrap ? w : 0u);
-      p += wrap ? bp : ap;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) e[k] += wrap ? past[k] : in_row[k];
-      s += step;
-    }
-    if constexpr (TEST) {
-      uint32_t z[N];
-#pragma unroll
-      for (int i = 0; i < N; ++i) z[i] = on[i] ? zkey(A, pix[i]) : 0u;
-#pragma unroll
-      for (int i = 0; i < N; ++i) hit |= on[i] && key[i] <= z[i];
+  const uint32_t w = (uint32_t)(px1 - px0 + 1), n = w * (uint32_t)(py1 - py0 + 1);
+  Put q;
+  for (uint32_t s = first; s < n; s += step) {
+    const int px = px0 + (int)(s % w), py = py0 + (int)(s / w);
+    const Edges E = edges_at(a, b, c, px, py);
+    const bool in = (E.e[0] > 0 || (E.e[0] == 0 && E.tl[0])) && (E.e[1] > 0 || (E.e[1] == 0 && E.tl[1])) &&
+                    (E.e[2] > 0 || (E.e[2] == 0 && E.tl[2]));
+    if (!in) continue;
+    float f = __fmul_rn(ll2float_rn(E.e[0]), a.zn);
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[1]), b.zn));
+    f = __fadd_rn(f, __fmul_rn(ll2float_rn(E.e[2]), c.zn));
+    const float d = __fmul_rn(f, invA);
+    if (!(d >= -1.0f && d <= 1.0f)) continue;
+    const uint32_t key = ordered(d), p = (uint32_t)py * (uint32_t)A.W + (uint32_t)px;
+    if (TEST) {
+      if (key <= zkey(A, p)) return true;
     } else {
-      later.put(A, t, on, key, pix);
+      q.put(A, p, key, t);
     }
   }
-  if constexpr (!TEST) later.check(A, t);
-  return hit;
+  if (!TEST) q.check(A, t);
+  return false;
 }
 
 // Record e of the queue: a large sub-triangle whose tiles are numbered from `tile` on.
@@ -1426,7 +1447,7 @@ __device__ __forceinline__ void own_tiles(const RasterArgs& A, uint32_t e, uint6
 
 // The record that tile g belongs to, the last one that starts at or before it: each round
 // the lanes look at 32 records evenly apart.
-__device__ __noinline__ uint32_t record_of(const RasterArgs& A, uint32_t n_ent, uint64_t g) {
+__device__ __forceinline__ uint32_t record_of(const RasterArgs& A, uint32_t n_ent, uint64_t g) {
   const uint32_t lane = threadIdx.x & 31;
   uint32_t lo = 0, hi = n_ent;
   while (hi - lo > 1u) {
@@ -1442,63 +1463,53 @@ __device__ __noinline__ uint32_t record_of(const RasterArgs& A, uint32_t n_ent, 
   return lo;
 }
 
-// Records of the queue and their tiles.  FULL: there may be more than the queue and the
-// owner table hold (tiles reserved past the last record belong to no one).
-struct Queued {
-  uint32_t records;
-  uint64_t tiles;
-};
-
-__device__ __forceinline__ bool overfull(const RasterArgs& A, unsigned long long st) {
-  return (st >> 40) > A.queue_cap || (st & ((1ull << 40) - 1)) > A.tile_cap;
-}
-
-template <bool FULL>
-__device__ __forceinline__ Queued queued(const RasterArgs& A, unsigned long long st) {
-  Queued n{(uint32_t)min(st >> 40, (unsigned long long)A.queue_cap), st & ((1ull << 40) - 1)};
-  if (FULL && (st >> 40) > A.queue_cap) {
-    const BigTri& q = A.queue[A.queue_cap - 1u];
-    n.tiles = first_tile(q.tile0, q.pad) + tiles_of(q.px1 - q.px0 + 1, q.py1 - q.py0 + 1);
-  }
-  return n;
-}
-
-// Tile::run(A, record, tile in it) for every tile of the queued records, a warp each.  The
-// table holds the owners of the first tile_cap tiles, four for each record there is room
-// for.  st: the queue's counter.  FULL: also the tiles past it (a few triangles that fill the view), in runs of
-// neighbours: the first one's record is looked up, the next ones' are the same or the next.
-// (Rasterized by the threads that set them up instead, 40 triangles that fill a 1080p
-// window take 1.7 s and 40 clipped ones 734 ms; so 0.69 and 0.33 ms.)
-template <class Tile, bool FULL>
+// Tile::run(A, record, tile in it) for every tile of the queued records, a warp each; st:
+// the queue's counter.  The table holds the owners of the first tile_cap tiles, four for
+// each record there is room for.  The tiles past it (of a few triangles that fill the
+// view) are taken in runs of neighbours: the first one's record is looked up, the next
+// ones' are the same or the next.  (Rasterized by the threads that set them up instead, 40
+// triangles that fill a 1080p window take 1.7 s and 40 clipped ones 734 ms; so 0.69 and
+// 0.33 ms.)
+template <class Tile>
 __device__ __forceinline__ void for_tiles(const RasterArgs& A, unsigned long long st, uint32_t bid, uint32_t nblk) {
   const uint32_t warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = (nblk * blockDim.x) >> 5;
-  const Queued n = queued<FULL>(A, st);
-  if (n.records == 0u) return;
-  const uint32_t n_tab = FULL ? (uint32_t)min(n.tiles, (uint64_t)A.tile_cap) : (uint32_t)n.tiles;
-  for (uint32_t g = warp; g < n_tab; g += nwarps) {
-    const BigTri& q = A.queue[__ldcg(A.tile_owner + g)];
-    Tile::run(A, q, g - q.tile0);
+  const uint32_t n_ent = (uint32_t)min((unsigned long long)A.queue_cap, st >> 40);
+  if (n_ent == 0u) return;
+  uint64_t n_tiles = st & ((1ull << 40) - 1);
+  if ((st >> 40) > A.queue_cap) {  // tiles reserved past the last record belong to no one
+    const BigTri& q = A.queue[n_ent - 1u];
+    n_tiles = first_tile(q.tile0, q.pad) + tiles_of(q.px1 - q.px0 + 1, q.py1 - q.py0 + 1);
   }
-  if (!FULL) return;
-  const uint64_t rest = n.tiles - n_tab, each = (rest + nwarps - 1u) / nwarps;
-  const uint32_t run = each > 32u ? 32u : (uint32_t)each;
-  for (uint64_t i = (uint64_t)warp * run; i < rest; i += (uint64_t)nwarps * run) {
-    uint64_t g = n_tab + i;
-    uint32_t e = record_of(A, n.records, g);
-    for (uint32_t k = (uint32_t)min((uint64_t)run, rest - i); k; --k, ++g) {
-      uint64_t local = g - first_tile(A.queue[e].tile0, A.queue[e].pad);
-      if (local >= tiles_of(A.queue[e].px1 - A.queue[e].px0 + 1, A.queue[e].py1 - A.queue[e].py0 + 1)) {
+  const uint32_t n_tab = (uint32_t)min(n_tiles, (uint64_t)A.tile_cap);
+  const uint64_t rest = n_tiles - n_tab, each = (rest + nwarps - 1u) / nwarps;
+  const uint32_t run = each < 1u ? 1u : each > 32u ? 32u : (uint32_t)each;
+  const uint64_t runs = (rest + run - 1u) / run;
+  for (uint64_t i = warp; i < n_tab + runs; i += nwarps) {
+    uint32_t e, k = 1u;
+    uint64_t g = i;
+    if (i < n_tab) {
+      e = __ldcg(A.tile_owner + i);
+    } else {
+      g = n_tab + (i - n_tab) * run;
+      k = (uint32_t)min((uint64_t)run, n_tiles - g);
+      e = record_of(A, n_ent, g);
+    }
+    for (; k; --k, ++g) {
+      const BigTri* q = A.queue + e;
+      uint64_t local = g - first_tile(q->tile0, q->pad);
+      if (local >= tiles_of(q->px1 - q->px0 + 1, q->py1 - q->py0 + 1)) {  // (the run's next record)
+        ++q;
         ++e;
         local = 0u;
       }
-      Tile::run(A, A.queue[e], (uint32_t)local);
+      Tile::run(A, *q, (uint32_t)local);
     }
   }
 }
 
-// A triangle that must be clipped (rare).  TEST as in win_rect64; else its sub-triangles
-// are rasterized here (small) or queued, their records first .. first + n - 1 returned
-// for their tiles' owners.
+// A triangle that must be clipped (rare).  Its sub-triangles are rasterized here (small,
+// or the queue is full) or queued, their records first .. first + n - 1 returned for their
+// tiles' owners.  TEST: those rasterized here, tested as in win_rect64.
 struct Fan {
   uint32_t first, n;
 };
@@ -1531,6 +1542,7 @@ __device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4
       tiles += tiles_of(w, h);
     }
   }
+  const bool full = TEST && (__ldcg(&A.ctr->big) >> 40) > A.queue_cap;
   uint64_t e = 0, tile = 0;
   if (nq) {
     const unsigned long long old = atomicAdd(&A.ctr->big, ((unsigned long long)nq << 40) | (unsigned long long)tiles);
@@ -1544,7 +1556,8 @@ __device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4
     const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
     if (s.A <= 0 || w <= 0 || h <= 0) continue;
     if (TEST) {
-      if (win_rect64<true>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u)) return true;
+      if ((w * h <= kSmallMaxPix || full) && win_rect64<true>(A, a, b, c, t, s.px0, s.py0, s.px1, s.py1, 0u, 1u))
+        return true;
       continue;
     }
     if (w * h > kSmallMaxPix) {
@@ -1575,6 +1588,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
   const uint32_t lane = threadIdx.x & 31;
   // (the clipped triangles' counts with the survivors': mostly there are none)
   uint32_t clipped = 0;
+  if (threadIdx.x == 0) *ties_full() = 0u;
 #pragma unroll
   for (uint32_t j = 0; j < (kMaxFrontBlocks + NT - 1) / NT; ++j)
     if (threadIdx.x + j * NT < A.front_blocks) clipped |= __ldcg(A.clip_count + threadIdx.x + j * NT);
@@ -1602,8 +1616,8 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
         if (kind == 2) tiles = tiles_of(w, h);
       }
     }
-    // large triangles of the warp reserve queue records and tiles with one atomic; a
-    // triangle that finds no record any more is listed as a mid-size one, whatever its size
+    // large triangles of the warp reserve queue records and tiles with one atomic; what
+    // finds no record any more is listed as mid-size, or, too large for 32 bits, done here
     const uint32_t bigs = __ballot_sync(0xFFFFFFFFu, kind == 2);
     if (bigs) {
       uint32_t tpre = tiles;  // inclusive prefix of tiles over the warp
@@ -1623,7 +1637,12 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
         win_queue(A, E.v.X, E.v.Y, E.v.z, E.px0, E.py0, E.px1, E.py1, E.fits, t, (uint32_t)e, tile);
       } else {
         tiles = 0;
-        if (kind == 2) kind = 3;
+        if (kind == 2 && E.fits) {
+          kind = 3;
+        } else if (kind == 2) {
+          const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
+          win_rect64<false>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
+        }
       }
       own_tiles(A, (uint32_t)e, tile, tiles);
     }
@@ -1638,8 +1657,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
           d[0] = make_float4(__int_as_float(E.v.X[0]), __int_as_float(E.v.Y[0]), __int_as_float(E.v.X[1]),
                              __int_as_float(E.v.Y[1]));
           d[1] = make_float4(__int_as_float(E.v.X[2]), __int_as_float(E.v.Y[2]),
-                             __int_as_float(E.px0 | (E.py0 << 16)),
-                             __int_as_float(E.px1 | (E.py1 << 16) | (E.fits ? 0 : (int)0x80000000)));
+                             __int_as_float(E.px0 | (E.py0 << 16)), __int_as_float(E.px1 | (E.py1 << 16)));
           d[2] = make_float4(E.v.z[0], E.v.z[1], E.v.z[2], __uint_as_float(t));
         } else {
           set_status(A.ctr, FA_E_CAPACITY);
@@ -1647,7 +1665,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
       }
     }
     if (!grouped) {
-      if (kind == 1) win_box<4>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
+      if (kind == 1) win_box<4, kPut>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
     } else {
       // the group's leader holds the triangle; each lane takes one sample of its box
       const uint32_t src = lane & ~(kRasterGroup - 1u);
@@ -1662,7 +1680,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
       const int px1 = __shfl_sync(0xFFFFFFFFu, E.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, E.py1, src);
       const uint32_t gt = __shfl_sync(0xFFFFFFFFu, t, src);
       const bool go = __shfl_sync(0xFFFFFFFFu, kind, src) == 1;
-      if (go) win_box<1>(A, g, gt, px0, py0, px1, py1, (int)sub, (int)kRasterGroup);
+      if (go) win_box<1, kPut>(A, g, gt, px0, py0, px1, py1, (int)sub, (int)kRasterGroup);
     }
   }
   // then the (rare) triangles that need clipping, from the front blocks' regions
@@ -1690,6 +1708,13 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
       own_tiles(A, fan.first + q, tile, tiles);
     }
   }
+}
+
+// Lanes (their log2) of each of n listed sub-triangles on a grid of `stride` threads.
+__device__ __forceinline__ uint32_t mid_lanes(uint32_t n, uint32_t stride) {
+  uint32_t lg = kMinLanes;
+  while (lg < 5u && ((uint64_t)n << (lg + 1u)) <= stride) ++lg;
+  return lg;
 }
 
 // The listed record of position i, pre: where each list starts.
@@ -1764,22 +1789,6 @@ struct PutTile {
   }
 };
 
-// The listed sub-triangles that found no queue record and are too large for 32 bits, a
-// warp each (rare).
-__device__ __forceinline__ void mid_wide(const RasterArgs& A, uint32_t bid, uint32_t nblk, const uint32_t* pre) {
-  const uint32_t n = pre[kMidLists], lane = threadIdx.x & 31;
-  for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> 5; i < n; i += (nblk * blockDim.x) >> 5) {
-    const float4* s = mid_record(A, pre, i);
-    const float4 f0 = __ldcg(s), f1 = __ldcg(s + 1), f2 = __ldcg(s + 2);
-    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
-    if ((int)b1 >= 0) continue;
-    const SV a{__float_as_int(f0.x), __float_as_int(f0.y), f2.x}, b{__float_as_int(f0.z), __float_as_int(f0.w), f2.y},
-        c{__float_as_int(f1.x), __float_as_int(f1.y), f2.z};
-    win_rect64<false>(A, a, b, c, __float_as_uint(f2.w), (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu),
-                      (int)((b1 >> 16) & 0x7FFFu), lane, 32u);
-  }
-}
-
 // Where each mid-size list starts, pre[0] .. pre[kMidLists] (seen after a barrier).
 __device__ __forceinline__ void mid_prefix(const RasterArgs& A, uint32_t* pre) {
   const uint32_t lane = threadIdx.x & 31;
@@ -1798,16 +1807,18 @@ __device__ __forceinline__ void mid_prefix(const RasterArgs& A, uint32_t* pre) {
   }
 }
 
-// The queued tiles, a warp each, then the mid-size lists.
-template <bool FULL>
-__device__ __forceinline__ void depth_win(const RasterArgs& A, unsigned long long st, uint32_t bid, uint32_t nblk,
-                                          uint32_t* pre) {
-  for_tiles<PutTile, FULL>(A, st, bid, nblk);
+// The queued tiles, a warp each, then the mid-size lists.  (No call of a function that is
+// not inlined: with one in a branch that is never taken the mid-size boxes of a
+// 3.2M-triangle floor take 440 us instead of 330.)
+__device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  __shared__ uint32_t pre[kMidLists + 1];
+  const unsigned long long st = __ldcg(&A.ctr->big);
+  if (threadIdx.x == 0) *ties_full() = 0u;
+  mid_prefix(A, pre);  // (a barrier)
+  for_tiles<PutTile>(A, st, bid, nblk);
   __syncthreads();
   const uint32_t n = pre[kMidLists], stride = nblk * blockDim.x;
-  uint32_t lg = kMinLanes;
-  while (lg < 5u && ((uint64_t)n << (lg + 1u)) <= stride) ++lg;
-  const uint32_t sub = threadIdx.x & ((1u << lg) - 1u);
+  const uint32_t lg = mid_lanes(n, stride), sub = threadIdx.x & ((1u << lg) - 1u);
   for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> lg; i < n; i += stride >> lg) {
     const float4* s = mid_record(A, pre, i);
     const float4 f0 = __ldcs(s), f1 = __ldcs(s + 1), f2 = __ldcs(s + 2);
@@ -1816,23 +1827,8 @@ __device__ __forceinline__ void depth_win(const RasterArgs& A, unsigned long lon
                   {f2.x, f2.y, f2.z}};
     const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w), t = __float_as_uint(f2.w);
     const int px0 = (int)(b0 & 0xFFFFu), py0 = (int)(b0 >> 16), px1 = (int)(b1 & 0xFFFFu), py1 = (int)(b1 >> 16);
-    if ((int)b1 >= 0) win_box<4, true>(A, v, t, px0, py0, px1, py1, (int)sub, 1 << lg);
+    win_box<4, kPutLater>(A, v, t, px0, py0, px1, py1, (int)sub, 1 << lg);
   }
-  if (FULL) mid_wide(A, bid, nblk, pre);
-}
-
-__device__ __noinline__ void depth_win_full(const RasterArgs& A, uint32_t bid, uint32_t nblk, uint32_t* pre) {
-  depth_win<true>(A, __ldcg(&A.ctr->big), bid, nblk, pre);
-}
-
-// (the full form on its own: in one body with the other it takes that one's registers,
-// and 60 patches at 1080p, which have no large triangle, 57 us instead of 39)
-__device__ __forceinline__ void depth_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
-  __shared__ uint32_t pre[kMidLists + 1];
-  const unsigned long long st = __ldcg(&A.ctr->big);
-  mid_prefix(A, pre);
-  if (overfull(A, st)) depth_win_full(A, bid, nblk, pre);
-  else depth_win<false>(A, st, bid, nblk, pre);
 }
 
 // Sets triangle t's visible bit.
@@ -1843,48 +1839,81 @@ __device__ __forceinline__ void win_mark(const RasterArgs& A, uint32_t t) {
   note_tile(A, t >> 10);
 }
 
-// The marking pass when the tie list overflowed: every survivor and clipped triangle
-// tested against the final keys.
+// Whether triangle t is marked.
+__device__ __forceinline__ bool marked(const RasterArgs& A, uint32_t t) {
+  return (__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u;
+}
+
+// A tile of the marking passes over the final keys.
+template <int PASS>
+struct MarkTile {
+  static __device__ __forceinline__ void run(const RasterArgs& A, const BigTri& q, uint32_t local) {
+    raster_tile<PASS, true>(A, q, local);
+  }
+};
+
+template <int PASS>
+__device__ __noinline__ void mark_tiles(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  for_tiles<MarkTile<PASS>>(A, __ldcg(&A.ctr->big), bid, nblk);
+}
+
+// The listed sub-triangles whose triangles are not marked, against the final keys.
+__device__ __noinline__ void mark_mids(const RasterArgs& A, uint32_t bid, uint32_t nblk, const uint32_t* pre) {
+  const uint32_t n = pre[kMidLists], stride = nblk * blockDim.x;
+  const uint32_t lg = mid_lanes(n, stride), sub = threadIdx.x & ((1u << lg) - 1u);
+  for (uint32_t i = (bid * blockDim.x + threadIdx.x) >> lg; i < n; i += stride >> lg) {
+    const float4* s = mid_record(A, pre, i);
+    const float4 f2 = __ldcs(s + 2);
+    const uint32_t t = __float_as_uint(f2.w);
+    if (marked(A, t)) continue;
+    const float4 f0 = __ldcs(s), f1 = __ldcs(s + 1);
+    const Tri32 v{{__float_as_int(f0.x), __float_as_int(f0.z), __float_as_int(f1.x)},
+                  {__float_as_int(f0.y), __float_as_int(f0.w), __float_as_int(f1.y)},
+                  {f2.x, f2.y, f2.z}};
+    const uint32_t b0 = __float_as_uint(f1.z), b1 = __float_as_uint(f1.w);
+    if (win_box<4, kTest>(A, v, t, (int)(b0 & 0xFFFFu), (int)(b0 >> 16), (int)(b1 & 0xFFFFu), (int)(b1 >> 16), (int)sub,
+                          1 << lg))
+      win_mark(A, t);
+  }
+}
+
+// The marking pass when the tie list overflowed: every sub-triangle whose triangle is not
+// marked is tested against the final keys, where the depth pass had it: the queued tiles,
+// the mid-size lists, the small ones from their survivors and their clipped fans.
 template <int NT>
 __device__ __noinline__ void mark_all(const RasterArgs& A, uint32_t bid, uint32_t nblk, uint32_t* pre) {
+  __shared__ uint32_t mid_pre[kMidLists + 1];
+  mid_prefix(A, mid_pre);
   const uint32_t lane = threadIdx.x & 31;
-  const uint32_t n = surv_prefix<NT>(A, pre);
+  const uint32_t n = surv_prefix<NT>(A, pre);  // (a barrier: mid_pre is written)
+  mark_tiles<1>(A, bid, nblk);
+  mark_mids(A, bid, nblk, mid_pre);
   const uint32_t stride = nblk * blockDim.x;
+  const bool full = (__ldcg(&A.ctr->big) >> 40) > A.queue_cap;
   for (uint32_t wbase = bid * blockDim.x + (threadIdx.x & ~31u); wbase < n; wbase += stride) {
     const uint32_t v = wbase + lane;
-    WinSetup E = {};
-    uint32_t t = 0;
-    bool vis = false, large = false;
-    if (v < n) {
-      const uint32_t i = surv_slot(A, pre, v, wbase);
-      const float4* sc = A.surv_clip + 3 * (size_t)i;
-      t = __ldcg(A.surv + i);
-      E = win_setup(A, sc[0], sc[1], sc[2]);
-      if (E.live) {
-        large = (E.px1 - E.px0 + 1) * (E.py1 - E.py0 + 1) > kMidPix;
-        const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
-        if (!large) vis = win_rect64<true>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
-      }
+    if (v >= n) continue;
+    const uint32_t i = surv_slot(A, pre, v, wbase);
+    const uint32_t t = __ldcg(A.surv + i);
+    if (marked(A, t)) continue;
+    const float4* sc = A.surv_clip + 3 * (size_t)i;
+    const WinSetup E = win_setup(A, __ldcs(sc), __ldcs(sc + 1), __ldcs(sc + 2));
+    if (!E.live) continue;
+    bool hit = false;
+    if (!E.fits) {  // (queued, unless there was no room)
+      const SV a{E.v.X[0], E.v.Y[0], E.v.z[0]}, b{E.v.X[1], E.v.Y[1], E.v.z[1]}, c{E.v.X[2], E.v.Y[2], E.v.z[2]};
+      hit = full && win_rect64<true>(A, a, b, c, t, E.px0, E.py0, E.px1, E.py1, 0u, 1u);
+    } else if ((E.px1 - E.px0 + 1) * (E.py1 - E.py0 + 1) <= kSmallMaxPix) {
+      hit = win_box<4, kTest>(A, E.v, t, E.px0, E.py0, E.px1, E.py1, 0, 1);
     }
-    for (uint32_t m = __ballot_sync(0xFFFFFFFFu, large); m; m &= m - 1u) {  // the warp together
-      const int src = __ffs(m) - 1;
-      SV q[3];
-#pragma unroll
-      for (int j = 0; j < 3; ++j)
-        q[j] = SV{__shfl_sync(0xFFFFFFFFu, E.v.X[j], src), __shfl_sync(0xFFFFFFFFu, E.v.Y[j], src),
-                  __shfl_sync(0xFFFFFFFFu, E.v.z[j], src)};
-      const int px0 = __shfl_sync(0xFFFFFFFFu, E.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, E.py0, src);
-      const int px1 = __shfl_sync(0xFFFFFFFFu, E.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, E.py1, src);
-      const bool hit = win_rect64<true>(A, q[0], q[1], q[2], 0u, px0, py0, px1, py1, lane, 32u);
-      if (__any_sync(0xFFFFFFFFu, hit) && (int)lane == src) vis = true;
-    }
-    if (vis) win_mark(A, t);
+    if (hit) win_mark(A, t);
   }
   __syncthreads();  // pre is reused
   const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
   const Mat4 M = A.Mdev ? load_mat(A.Mdev) : A.M;
   for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
     const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
+    if (marked(A, t)) continue;
     const uint32_t* f = A.idx + 3 * (size_t)t;
     Fan fan;
     if (win_clipped<true>(A, t, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
@@ -1953,17 +1982,20 @@ __device__ __forceinline__ void mark_win_body(const RasterArgs& A, uint32_t bid,
       note_tile(A, tile);
     }
   }
+  if (s_ties > kTies) {
+    // (conservative marking tests what is not marked anyway; the blocks of the first wave
+    // alone, so that no share of the tests waits for the second)
+    const uint32_t share = min(nblk, kMarkBlocks);
+    if (!A.cons && bid < share) mark_all<NT>(A, bid, share, pre);
+    return;
+  }
   const uint32_t stride = nblk * blockDim.x;
-  if (s_ties <= A.tie_cap) {
-    for (uint32_t i = bid * blockDim.x + threadIdx.x; i < s_ties; i += stride) {
-      const uint4 e = __ldcg(A.ties + i);
-      if (zkey(A, e.x) == e.y) {
-        win_mark(A, e.z);
-        win_mark(A, e.w);
-      }
+  for (uint32_t i = bid * blockDim.x + threadIdx.x; i < s_ties; i += stride) {
+    const uint4 e = __ldcg(A.ties + i);
+    if (zkey(A, e.x) == e.y) {
+      win_mark(A, e.z);
+      win_mark(A, e.w);
     }
-  } else {
-    mark_all<NT>(A, bid, nblk, pre);
   }
 }
 
@@ -2139,7 +2171,6 @@ inline RasterArgs make_raster_args(fa_ctx* ctx, const fa_mesh* mesh, const Mat4&
   A.vt = vt;
   A.zid = reinterpret_cast<unsigned long long*>(ctx->zbuf);
   A.ties = ctx->ties;
-  A.tie_cap = ctx->tie_cap;
   set_raster_mode(A);
   return A;
 }
