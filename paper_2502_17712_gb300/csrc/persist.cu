@@ -126,9 +126,9 @@ template <bool DEV_M>
 __device__ __noinline__ void st_exact(const ViewArgs& v, uint32_t j, uint32_t n) {
   rs::exact_body<DEV_M, kPT>(v.ra, j, n);
 }
-template <bool DEV_M>
+template <bool DEV_M, bool CONS>
 __device__ __noinline__ void st_exact_win(const ViewArgs& v, uint32_t j, uint32_t n) {
-  rs::exact_win_body<DEV_M, kPT>(v.ra, j, n);
+  rs::exact_win_body<DEV_M, kPT, CONS>(v.ra, j, n);
 }
 __device__ __noinline__ void st_depth_big(const ViewArgs& v, uint32_t j, uint32_t n) { rs::depth_big_body(v.ra, j, n); }
 __device__ __noinline__ void st_depth_win(const ViewArgs& v, uint32_t j, uint32_t n) { rs::depth_win_body(v.ra, j, n); }
@@ -203,7 +203,7 @@ __device__ __forceinline__ void run_stage_inline(const ViewArgs& v, uint32_t sta
   // (the device-matrix and conservative variants, and the other stages, keep their
   // own register allocation in the non-inlined wrappers)
   if (stage == S_FRONT && !v.devm) rs::front_body<false>(v.ra, j, n);
-  else if (stage == S_EXACT && !v.devm && v.ra.win) rs::exact_win_body<false, kPT>(v.ra, j, n);
+  else if (stage == S_EXACT && !v.devm && v.ra.win && !v.cons) rs::exact_win_body<false, kPT, false>(v.ra, j, n);
   else if (stage == S_DEPTH_BIG && v.ra.win) rs::depth_win_body(v.ra, j, n);
   else run_stage(v, stage, j, n, smem);
 }
@@ -212,7 +212,8 @@ __device__ void run_stage(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_
   switch (stage) {
     case S_FRONT: v.devm ? st_front<true>(v, j, n) : st_front<false>(v, j, n); break;
     case S_EXACT:
-      if (v.ra.win) v.devm ? st_exact_win<true>(v, j, n) : st_exact_win<false>(v, j, n);
+      if (v.ra.win && v.cons) v.devm ? st_exact_win<true, true>(v, j, n) : st_exact_win<false, true>(v, j, n);
+      else if (v.ra.win) v.devm ? st_exact_win<true, false>(v, j, n) : st_exact_win<false, false>(v, j, n);
       else v.devm ? st_exact<true>(v, j, n) : st_exact<false>(v, j, n);
       break;
     case S_DEPTH_BIG: v.ra.win ? st_depth_win(v, j, n) : st_depth_big(v, j, n); break;

@@ -16,10 +16,13 @@ __global__ void __launch_bounds__(rs::kFrontThreads, 2) k_raster_front(RasterArg
   rs::front_body<DEV_M>(A, blockIdx.x, gridDim.x);
 }
 
-template <bool DEV_M, bool WIN>
+enum ExactMode { kExactTwice, kExactWinners, kExactWinnersCons };
+
+template <bool DEV_M, int MODE>
 __global__ void __launch_bounds__(256, 4) k_raster_exact(RasterArgs A) {
   pdl_wait();
-  if (WIN) rs::exact_win_body<DEV_M, 256>(A, blockIdx.x, gridDim.x);
+  if (MODE == kExactWinners) rs::exact_win_body<DEV_M, 256, false>(A, blockIdx.x, gridDim.x);
+  else if (MODE == kExactWinnersCons) rs::exact_win_body<DEV_M, 256, true>(A, blockIdx.x, gridDim.x);
   else rs::exact_body<DEV_M, 256>(A, blockIdx.x, gridDim.x);
 }
 
@@ -73,10 +76,12 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
   else
     launch_k(k_raster_front<false>, A.front_blocks, rs::kFrontThreads, 0, s, A);
   mark(ctx, "k_raster_exact", s);
-  if (A.win)
-    launch_k(Mdev ? k_raster_exact<true, true> : k_raster_exact<false, true>, gb, 256, 0, s, A);
+  if (A.win && cons)
+    launch_k(Mdev ? k_raster_exact<true, kExactWinnersCons> : k_raster_exact<false, kExactWinnersCons>, gb, 256, 0, s, A);
+  else if (A.win)
+    launch_k(Mdev ? k_raster_exact<true, kExactWinners> : k_raster_exact<false, kExactWinners>, gb, 256, 0, s, A);
   else
-    launch_k(Mdev ? k_raster_exact<true, false> : k_raster_exact<false, false>, gb, 256, 0, s, A);
+    launch_k(Mdev ? k_raster_exact<true, kExactTwice> : k_raster_exact<false, kExactTwice>, gb, 256, 0, s, A);
   mark(ctx, "k_raster_depth_big", s);
   launch_k(A.win ? k_raster_depth_big<true> : k_raster_depth_big<false>, gb, 256, 0, s, A);
   if (A.zmax) {

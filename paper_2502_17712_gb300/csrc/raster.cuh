@@ -1138,7 +1138,8 @@ struct WinSetup {
   Tri32 v;
   int px0, py0, px1, py1;
   bool fits;  // 32-bit edge functions
-  bool live;  // front facing, with a sample in its box
+  bool front;  // front facing
+  bool live;   // front facing, with a sample in its box
 };
 
 __device__ __forceinline__ uint32_t tiles_of(int w, int h) {
@@ -1173,9 +1174,26 @@ __device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4&
   s.py1 = min((ymx - 128) >> 8, A.H - 1);
   s.fits = fits32(s.v);
   const int ux = s.v.X[1] - s.v.X[0], uy = s.v.Y[1] - s.v.Y[0], vx = s.v.X[2] - s.v.X[0], vy = s.v.Y[2] - s.v.Y[0];
-  const bool front = s.fits ? ux * vy - vx * uy > 0 : (int64_t)ux * vy - (int64_t)vx * uy > 0;
-  s.live = front && s.px1 >= s.px0 && s.py1 >= s.py0;
+  s.front = s.fits ? ux * vy - vx * uy > 0 : (int64_t)ux * vy - (int64_t)vx * uy > 0;
+  s.live = s.front && s.px1 >= s.px0 && s.py1 >= s.py0;
   return s;
+}
+
+// Conservative marking takes a sub-triangle whose conservative box has more than kMidPix
+// pixels by tiles, so the exact pass queues it with that box (as setup's; the samples past
+// its own box are not covered).  Gives s that box if so.
+__device__ __forceinline__ bool cons_queue(const RasterArgs& A, WinSetup& s) {
+  if (!s.front) return false;
+  const int xmn = min(s.v.X[0], min(s.v.X[1], s.v.X[2])), xmx = max(s.v.X[0], max(s.v.X[1], s.v.X[2]));
+  const int ymn = min(s.v.Y[0], min(s.v.Y[1], s.v.Y[2])), ymx = max(s.v.Y[0], max(s.v.Y[1], s.v.Y[2]));
+  const int px0 = max(-((-xmn) >> 8) - 1, 0), px1 = min(xmx >> 8, A.W - 1);
+  const int py0 = max(-((-ymn) >> 8) - 1, 0), py1 = min(ymx >> 8, A.H - 1);
+  if (px1 < px0 || py1 < py0 || (px1 - px0 + 1) * (py1 - py0 + 1) <= kMidPix) return false;
+  s.px0 = px0;
+  s.py0 = py0;
+  s.px1 = px1;
+  s.py1 = py1;
+  return true;
 }
 
 // Set once this block has found the tie list full (cleared before a pass's first sample).
@@ -1535,7 +1553,7 @@ __device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4
   for (int i = 0; i < n; ++i) sv[i] = project(poly[i], A.hx, A.hy);
   if (!TEST) {
     for (int i = 1; i + 1 < n; ++i) {
-      const Setup s = setup(sv[0], sv[i], sv[i + 1], A.W, A.H, false);
+      const Setup s = setup(sv[0], sv[i], sv[i + 1], A.W, A.H, A.cons);
       const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
       if (s.A <= 0 || w <= 0 || h <= 0 || w * h <= kSmallMaxPix) continue;
       ++nq;
@@ -1552,7 +1570,7 @@ __device__ __noinline__ bool win_clipped(const RasterArgs& A, uint32_t t, float4
   }
   for (int i = 1; i + 1 < n; ++i) {
     const SV &a = sv[0], &b = sv[i], &c = sv[i + 1];
-    const Setup s = setup(a, b, c, A.W, A.H, false);
+    const Setup s = setup(a, b, c, A.W, A.H, A.cons);
     const int w = s.px1 - s.px0 + 1, h = s.py1 - s.py0 + 1;
     if (s.A <= 0 || w <= 0 || h <= 0) continue;
     if (TEST) {
@@ -1582,7 +1600,8 @@ __device__ __forceinline__ uint32_t mid_base(const RasterArgs& A, uint32_t r) {
 
 // Exact set-up of the survivors (as exact_body): small ones rasterized here, mid-size
 // ones listed, large ones queued.
-template <bool DEV_M, int NT>
+// CONS: for conservative marking (cons_queue).
+template <bool DEV_M, int NT, bool CONS>
 __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
   uint32_t* pre = region_pre();
   const uint32_t lane = threadIdx.x & 31;
@@ -1613,8 +1632,9 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
       if (E.live) {
         const int w = E.px1 - E.px0 + 1, h = E.py1 - E.py0 + 1, pix = w * h;
         kind = !E.fits ? 2 : pix <= kSmallMaxPix ? 1 : pix <= kMidPix ? 3 : 2;
-        if (kind == 2) tiles = tiles_of(w, h);
       }
+      if (CONS && cons_queue(A, E)) kind = 2;
+      if (kind == 2) tiles = tiles_of(E.px1 - E.px0 + 1, E.py1 - E.py0 + 1);
     }
     // large triangles of the warp reserve queue records and tiles with one atomic; what
     // finds no record any more is listed as mid-size, or, too large for 32 bits, done here
@@ -1852,9 +1872,8 @@ struct MarkTile {
   }
 };
 
-template <int PASS>
 __device__ __noinline__ void mark_tiles(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
-  for_tiles<MarkTile<PASS>>(A, __ldcg(&A.ctr->big), bid, nblk);
+  for_tiles<MarkTile<1>>(A, __ldcg(&A.ctr->big), bid, nblk);
 }
 
 // The listed sub-triangles whose triangles are not marked, against the final keys.
@@ -1886,7 +1905,7 @@ __device__ __noinline__ void mark_all(const RasterArgs& A, uint32_t bid, uint32_
   mid_prefix(A, mid_pre);
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t n = surv_prefix<NT>(A, pre);  // (a barrier: mid_pre is written)
-  mark_tiles<1>(A, bid, nblk);
+  mark_tiles(A, bid, nblk);
   mark_mids(A, bid, nblk, mid_pre);
   const uint32_t stride = nblk * blockDim.x;
   const bool full = (__ldcg(&A.ctr->big) >> 40) > A.queue_cap;
@@ -2002,8 +2021,11 @@ __device__ __forceinline__ void mark_win_body(const RasterArgs& A, uint32_t bid,
 // Conservative marking after the winners': the triangles that the samples marked are
 // marked already (a covered centre's depth is the sample's), so only the other survivors
 // are tested, each pixel of their conservative boxes against the final keys (as
-// sample<2>).  With many survivors, boxes of at most kSmallMaxPix pixels in-thread and
-// larger ones by the warp together; with few, a warp takes few of them, all together.
+// sample<2>).  Boxes above kMidPix pixels and clipped triangles' are the queued tiles, a warp
+// each, as in two rasterizations: a hidden triangle is looked at whole, and one that fills
+// a 1080p window takes a warp 18 ms and, clipped, a thread 0.77 s (by tiles 29 and 33 us).  Of the others
+// those of at most kSmallMaxPix pixels are tested in-thread and larger ones by the warp
+// together when there are many survivors; with few, a warp takes few of them, all together.
 // Against a second rasterization of every survivor (conservative fa_visibility at 1080p):
 // a floor of 60 patches 387 -> 250 us, 200 icospheres 209 -> 183.  What is left is the
 // hidden triangles' boxes, every pixel of them; four pixels' loads at once cost
@@ -2036,8 +2058,8 @@ __device__ __forceinline__ bool cons_box(const RasterArgs& A, const SV& a, const
   return false;
 }
 
-// The sub-triangles of a triangle that must be clipped (rare).
-__device__ __noinline__ bool cons_clipped(const RasterArgs& A, float4 c0, float4 c1, float4 c2) {
+// The sub-triangles of a triangle that must be clipped (rare) that are not queued.
+__device__ __noinline__ bool cons_clipped(const RasterArgs& A, float4 c0, float4 c1, float4 c2, bool full) {
   CV poly[kMaxPoly];
   poly[0] = CV{c0.x, c0.y, c0.z, c0.w};
   poly[1] = CV{c1.x, c1.y, c1.z, c1.w};
@@ -2051,6 +2073,7 @@ __device__ __noinline__ bool cons_clipped(const RasterArgs& A, float4 c0, float4
   for (int i = 1; i + 1 < n; ++i) {
     const Setup s = setup(sv[0], sv[i], sv[i + 1], A.W, A.H, true);
     if (s.A <= 0 || s.px1 < s.px0 || s.py1 < s.py0) continue;
+    if (!full && (s.px1 - s.px0 + 1) * (s.py1 - s.py0 + 1) > kSmallMaxPix) continue;
     if (cons_box(A, sv[0], sv[i], sv[i + 1], s.px0, s.py0, s.px1, s.py1, 0u, 1u)) return true;
   }
   return false;
@@ -2064,6 +2087,9 @@ __device__ __forceinline__ void mark_cons_body(const RasterArgs& A, uint32_t bid
   if (threadIdx.x == 0) s_cons_status = __ldcg(&A.ctr->status);
   __syncthreads();
   if (s_cons_status != 0) return;
+  // (a queue that has no more room: large ones that found no record are tested here)
+  const bool full = (__ldcg(&A.ctr->big) >> 40) > A.queue_cap;
+  const int most = full ? 0x7FFFFFFF : kMidPix;
   const uint32_t lane = threadIdx.x & 31;
   const uint32_t n = surv_prefix<NT>(A, pre);
   const uint32_t stride = nblk * blockDim.x, warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = stride >> 5;
@@ -2085,8 +2111,9 @@ __device__ __forceinline__ void mark_cons_body(const RasterArgs& A, uint32_t bid
         b = project(CV{c1.x, c1.y, c1.z, c1.w}, A.hx, A.hy);
         c = project(CV{c2.x, c2.y, c2.z, c2.w}, A.hx, A.hy);
         S = setup(a, b, c, A.W, A.H, true);
-        if (S.A > 0 && S.px1 >= S.px0 && S.py1 >= S.py0) {
-          big = (S.px1 - S.px0 + 1) * (S.py1 - S.py0 + 1) > (per < 32u ? 1 : kSmallMaxPix);
+        const int pix = (S.px1 - S.px0 + 1) * (S.py1 - S.py0 + 1);
+        if (S.A > 0 && S.px1 >= S.px0 && S.py1 >= S.py0 && pix <= most) {
+          big = pix > (per < 32u ? 1 : kSmallMaxPix);
           if (!big) vis = cons_box(A, a, b, c, S.px0, S.py0, S.px1, S.py1, 0u, 1u);
         }
       }
@@ -2114,9 +2141,11 @@ __device__ __forceinline__ void mark_cons_body(const RasterArgs& A, uint32_t bid
     if ((__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u) continue;
     const uint32_t* f = A.idx + 3 * (size_t)t;
     if (cons_clipped(A, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
-                     load_clip(M, A.pos, __ldg(f + 2))))
+                     load_clip(M, A.pos, __ldg(f + 2)), full))
       win_mark(A, t);
   }
+  // (inlined: as a call it takes the loops' registers, 60 patches at 1080p 244 us instead of 182)
+  for_tiles<MarkTile<2>>(A, __ldcg(&A.ctr->big), bid, nblk);
 }
 
 inline void set_raster_mode(RasterArgs& A);
