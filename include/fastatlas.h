@@ -60,7 +60,9 @@ typedef enum {
   FA_SELECT_LARGEST_K = 1  /* largest fitting candidate k (Sec. 4.2 literal)         */
 } fa_select_mode;
 
-/* Context maxima.  Scratch is sized from these once, in fa_create. */
+/* Context maxima.  Scratch is sized from these once, in fa_create.  The largest viewport's
+ * depth buffer takes 8 bytes a pixel; it shares its memory with the chart and pack scratch
+ * (about 1.1 KB a chart and 4 bytes a triangle and vertex), the larger of the two counts. */
 typedef struct {
   uint32_t max_tris;       /* triangles of the largest registered mesh              */
   uint32_t max_verts;      /* vertices of the largest registered mesh               */

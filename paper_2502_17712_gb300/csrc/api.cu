@@ -148,7 +148,6 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
   const uint64_t nblocks = (T + 1023) / 1024 + 1;
   Arena arena;
   arena.part(&ctx->ctr, (size_t)(1));
-  arena.part(&ctx->zbuf, (size_t)(2ull * c.max_width * c.max_height));
   arena.part(&ctx->zmax, (size_t)((uint64_t)((c.max_width + 15) / 16) * ((c.max_height + 15) / 16)));
   arena.part(&ctx->queue, (size_t)(ctx->queue_cap));
   ctx->tile_cap = 4u * ctx->queue_cap;
@@ -163,7 +162,6 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
   arena.part((float4**)&ctx->surv_clip, (size_t)ctx->surv_cap * 3);
   arena.part(&ctx->clip, (size_t)(ctx->surv_cap));
   arena.part(&ctx->clip_count, (size_t)(fa::kMaxFrontBlocks));
-  arena.part(&ctx->label, (size_t)(T + V));
   arena.part(&ctx->wordroots, (size_t)((T + 31) / 32));
   arena.part(&ctx->blockcnt, (size_t)(nblocks + 1));
   arena.part(&ctx->viscnt, (size_t)(nblocks + 1));
@@ -176,23 +174,29 @@ fa_status fa_create(fa_ctx** out, const fa_config* cfg) {
   arena.part(&pk.ord_rank, (size_t)(C));
   arena.part(&pk.ord_total, (size_t)(kMaxH));
   arena.part(&pk.order, (size_t)(C));
+  arena.part(&pk.scan_state, (size_t)((uint64_t)kMaxScales * pk.max_chunks));
+  arena.part(&pk.m, (size_t)(kMaxScales));
+  arena.part(&pk.cand, (size_t)(kMaxScales));
+  arena.part(&ctx->psched, (size_t)(kPschedWords));
+  // the depth buffer (8 bytes a pixel) and the ties, last read by the marking passes, share
+  // their memory with what the chart and pack passes after them write first
+  const size_t shared_from = arena.bytes;
+  arena.part(&ctx->ties, (size_t)kTies);
+  arena.part(&ctx->zbuf, (size_t)(2ull * c.max_width * c.max_height));
+  const size_t raster_end = arena.bytes;
+  arena.bytes = shared_from;
+  arena.part(&ctx->label, (size_t)(T + V));
   arena.part(&pk.fs, (size_t)((uint64_t)pk.max_chunks * kChunk));
   arena.part(&pk.rec8, (size_t)((uint64_t)kMaxScales * pk.max_chunks * kChunk));
   arena.part(&pk.segs, (size_t)((uint64_t)kMaxScales * pk.max_chunks * kSegStride));
-  arena.part(&pk.scan_state, (size_t)((uint64_t)kMaxScales * pk.max_chunks));
-  arena.part(&pk.m, (size_t)(kMaxScales));
   arena.part(&pk.xy, (size_t)((uint64_t)kMaxScales * C));
-  arena.part(&pk.cand, (size_t)(kMaxScales));
-  arena.part(&ctx->psched, (size_t)(kPschedWords));
+  arena.bytes = std::max(arena.bytes, raster_end);
   fa_status st = arena.place(&ctx->arena);
   if (st == FA_OK) {
     // the chart passes' edges and visible list lie where the raster's clip coordinates
-    // were (last read by the marking pass), the raster's ties where the push records will be
+    // were (last read by the marking passes)
     ctx->xedge = static_cast<uint2*>(ctx->surv_clip);
     ctx->vis = ctx->xedge + nblocks * 3072;
-    ctx->ties = reinterpret_cast<uint4*>(pk.rec8);
-    static_assert(kTies * sizeof(uint4) <= (uint64_t)kMaxScales * kChunk * sizeof(uint2),
-                  "the ties fit the push records of one chunk");
   }
   pk.ctr = ctx->ctr;
   pk.count = nullptr;

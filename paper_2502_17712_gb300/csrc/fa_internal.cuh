@@ -120,8 +120,8 @@ struct fa_ctx {
   // scratch, all of it in one allocation
   void* arena;
   fa::DevCounters* ctr;
-  uint32_t* zbuf;        // [max_w * max_h] depth keys, or 64-bit key | triangle
-  uint4* ties;           // [kTies] pixels where two triangles have the same key (in pack.rec8)
+  uint32_t* zbuf;        // [max_w * max_h] depth keys, or 64-bit key | triangle (in label .. pack.xy)
+  uint4* ties;           // [kTies] pixels where two triangles have the same key (likewise)
   uint32_t* zmax;        // [ceil(max_w / 16) * ceil(max_h / 16)] largest depth key per 16x16 tile
   uint32_t* tile_flag;   // [ceil(max_tris / 1024)] tile has a visible triangle (this frame)
   uint32_t* tile_list;   // [ceil(max_tris / 1024)] those tiles, in the order the marking found them
