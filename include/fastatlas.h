@@ -485,8 +485,8 @@ fa_status fa_batch_get_schedule(const fa_batch* batch, uint32_t* lanes, uint32_t
 fa_status fa_atlas_batch(fa_batch* batch, uint32_t n_views, const fa_mesh* const* meshes,
                          const fa_frame_params* params, const fa_frame_out* outs, fa_stream_t stream);
 
-/* Schedule autotuner: first the raster schedule of every lane's context (mid-size
- * limit 16 or 64, with and without FA_RASTER_HIZ, at the current lanes), then the
+/* Schedule autotuner: first the raster schedule of every lane's context (without
+ * FA_RASTER_HIZ, and with it at mid-size limits 16 and 64, at the current lanes), then the
  * chart/pack kernel shapes (uf_threads x push_threads in {256, 512, 1024}^2), then
  * lanes in {1, 2, 4, .., n_lanes} x both policies: each schedule's batch is captured into
  * a CUDA graph, launched once, `reps` launches are timed (CUDA events, best of) and
@@ -553,8 +553,8 @@ fa_status fa_batch_plan_get_schedule(const fa_batch_plan* plan, fa_plan_schedule
 fa_status fa_batch_plan_set_schedule(fa_batch_plan* plan, const fa_plan_schedule* schedule);
 
 /* Schedule autotuner: lanes in {1, 2, 4, .., n_lanes} x both policies x worker
- * counts at 50 / 100 / 200 %, after the raster schedule (mid-size limit 16 or 64,
- * with and without FA_RASTER_HIZ) was picked on all lanes; each schedule is
+ * counts at 50 / 100 / 200 %, after the raster schedule (without FA_RASTER_HIZ, and
+ * with it at mid-size limits 16 and 64) was picked on all lanes; each schedule is
  * launched once, then `reps` launches are timed (CUDA events, best of); the
  * fastest is kept.  Runs the views (outputs
  * are overwritten) and synchronizes; not for use inside a capture.  *best_ms (may

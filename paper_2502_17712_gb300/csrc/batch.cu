@@ -246,9 +246,10 @@ fa_status fa_batch_tune(fa_batch* b, uint32_t n_views, const fa_mesh* const* mes
   // the raster schedule first (at the current lanes, policy and kernel shapes), then
   // the chart/pack kernel shapes, then lanes x policy
   const uint32_t l0 = b->active, p0 = b->policy, u0 = best_u, q0 = best_q;
-  const uint32_t mids[] = {FA_RASTER_MID_OFF, 64};
-  for (uint32_t mid : mids)
-    for (uint32_t fl = 0; fl <= FA_RASTER_HIZ; ++fl) trial(l0, p0, mid, fl, u0, q0);
+  // (the mid-size limit belongs to the second rasterization, which only FA_RASTER_HIZ does)
+  trial(l0, p0, FA_RASTER_MID_OFF, 0, u0, q0);
+  trial(l0, p0, FA_RASTER_MID_OFF, FA_RASTER_HIZ, u0, q0);
+  trial(l0, p0, 64, FA_RASTER_HIZ, u0, q0);
   const uint32_t rm = best_m, rf = best_f;
   const uint32_t shapes[] = {256, 512, 1024};
   for (uint32_t uf : shapes)

@@ -805,10 +805,10 @@ fa_status fa_batch_plan_tune(fa_batch_plan* pl, uint32_t reps, float* best_ms) {
   // the raster schedule first (at the plan's lanes, policy and worker counts), then
   // lanes x policy x worker counts with the best raster schedule
   const fa_plan_schedule start = pl->sched;
-  const uint32_t mids[] = {FA_RASTER_MID_OFF, 64};
-  for (uint32_t mid : mids)
-    for (uint32_t fl = 0; fl <= FA_RASTER_HIZ; ++fl) trial(fa_plan_schedule{start.lanes, start.policy,
-                                                                             start.worker_pct, mid, fl});
+  // (the mid-size limit belongs to the second rasterization, which only FA_RASTER_HIZ does)
+  trial(fa_plan_schedule{start.lanes, start.policy, start.worker_pct, FA_RASTER_MID_OFF, 0});
+  trial(fa_plan_schedule{start.lanes, start.policy, start.worker_pct, FA_RASTER_MID_OFF, FA_RASTER_HIZ});
+  trial(fa_plan_schedule{start.lanes, start.policy, start.worker_pct, 64, FA_RASTER_HIZ});
   const uint32_t best_mid = best.mid_max_pix, best_fl = best.raster_flags;
   const uint32_t pcts[] = {50, 100, 200};
   for (uint32_t l : lanes)
