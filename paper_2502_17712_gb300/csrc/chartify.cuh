@@ -460,11 +460,9 @@ __device__ void scan_counts(uint32_t* a, uint32_t* b, uint32_t n, uint32_t* ta, 
     const uint4 x = load4(a, i, n);
     v.x += x.x + x.y + x.z + x.w;
     if (i == i0) a0 = x;
-    if (b) {
-      const uint4 y = load4(b, i, n);
-      v.y += y.x + y.y + y.z + y.w;
-      if (i == i0) b0 = y;
-    }
+    const uint4 y = load4(b, i, n);
+    v.y += y.x + y.y + y.z + y.w;
+    if (i == i0) b0 = y;
   }
   uint2 x = v;
 #pragma unroll
@@ -494,15 +492,13 @@ __device__ void scan_counts(uint32_t* a, uint32_t* b, uint32_t n, uint32_t* ta, 
   uint32_t ra = wp.x + x.x - v.x, rb = wp.y + x.y - v.y;
   for (uint32_t i = i0; i < i0 + per && i < n; i += 4u) {
     store4(a, i, n, excl4(i == i0 ? a0 : load4(a, i, n), ra));
-    if (b) store4(b, i, n, excl4(i == i0 ? b0 : load4(b, i, n), rb));
+    store4(b, i, n, excl4(i == i0 ? b0 : load4(b, i, n), rb));
   }
   if (threadIdx.x == 1023) {
     a[n] = wp.x + x.x;
     *ta = wp.x + x.x;
-    if (b) {
-      b[n] = wp.y + x.y;
-      *tb = wp.y + x.y;
-    }
+    b[n] = wp.y + x.y;
+    *tb = wp.y + x.y;
   }
   __syncthreads();
 }

@@ -896,7 +896,6 @@ __device__ __forceinline__ void exact_body(const RasterArgs& A, uint32_t bid, ui
 // from below.
 __device__ __forceinline__ bool hidden_by_tiles(const RasterArgs& A, float z0, float z1, float z2, int px0, int py0,
                                                 int px1, int py1) {
-  if (!A.zmax) return false;
   const float zmin = fminf(z0, fminf(z1, z2));
   const float zabs = fmaxf(fabsf(z0), fmaxf(fabsf(z1), fabsf(z2)));
   const float lo = __fsub_rd(zmin, __fmaf_ru(zabs, 1e-6f, 1e-37f));
