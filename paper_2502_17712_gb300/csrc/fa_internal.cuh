@@ -52,6 +52,7 @@ struct DevCounters {
   uint32_t n_vtiles;       // 1024-triangle tiles with a visible triangle (listed by the marking pass)
   uint32_t uf_item;        // next listed tile of the local union-find
   uint32_t n_ties;         // equal depth keys listed by the depth pass
+  uint32_t cons_item;      // next share of the conservative marking
   uint32_t n_mid[kMidLists][32];  // [.][0]: mid-size sub-triangles of each list (a line each)
 };
 

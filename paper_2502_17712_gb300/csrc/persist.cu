@@ -143,6 +143,9 @@ __device__ __noinline__ void st_mark_win(const ViewArgs& v, uint32_t j, uint32_t
 __device__ __noinline__ void st_mark_cons(const ViewArgs& v, uint32_t j, uint32_t n) {
   rs::mark_cons_body<kPT>(v.ra, j, n);
 }
+__device__ __noinline__ void st_mark_cons_tiles(const ViewArgs& v, uint32_t j, uint32_t n) {
+  rs::mark_cons_tiles(v.ra, j, n);
+}
 __device__ __noinline__ void st_init_v(const ViewArgs& v, uint32_t j, uint32_t n) {
   cf::init_v_body(v.uf.label, v.uf.T, v.uf.V, j, n);
 }
@@ -200,10 +203,10 @@ __device__ void run_stage(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_
 
 __device__ __forceinline__ void run_stage_inline(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_t n,
                                                  unsigned char* smem) {
-  // (the device-matrix and conservative variants, and the other stages, keep their
-  // own register allocation in the non-inlined wrappers)
+  // (the device-matrix variants and the other stages keep their own register allocation
+  // in the non-inlined wrappers)
   if (stage == S_FRONT && !v.devm) rs::front_body<false>(v.ra, j, n);
-  else if (stage == S_EXACT && !v.devm && v.ra.win && !v.cons) rs::exact_win_body<false, kPT, false>(v.ra, j, n);
+  else if (stage == S_EXACT && !v.devm && v.ra.win) rs::exact_win_body<false, kPT, true>(v.ra, j, n);
   else if (stage == S_DEPTH_BIG && v.ra.win) rs::depth_win_body(v.ra, j, n);
   else run_stage(v, stage, j, n, smem);
 }
@@ -219,7 +222,10 @@ __device__ void run_stage(const ViewArgs& v, uint32_t stage, uint32_t j, uint32_
     case S_DEPTH_BIG: v.ra.win ? st_depth_win(v, j, n) : st_depth_big(v, j, n); break;
     case S_ZMAX: st_zmax(v, j, n); break;
     case S_MARK: v.ra.win ? st_mark_win(v, j, n) : v.cons ? st_mark<true>(v, j, n) : st_mark<false>(v, j, n); break;
-    case S_MARK_CONS: st_mark_cons(v, j, n); break;
+    case S_MARK_CONS:
+      st_mark_cons(v, j, n);
+      st_mark_cons_tiles(v, j, n);
+      break;
     case S_INIT_V: st_init_v(v, j, n); break;
     case S_LOCAL: st_local(v, j, n); break;
     case S_HOOK: st_hook(v, j, n); break;

@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(256, 4) k_raster_mark(RasterArgs A) {
 __global__ void __launch_bounds__(256, 4) k_raster_mark_cons(RasterArgs A) {
   pdl_wait();
   rs::mark_cons_body<256>(A, blockIdx.x, gridDim.x);
+  rs::mark_cons_tiles(A, blockIdx.x, gridDim.x);
 }
 
 }  // namespace
@@ -97,7 +98,7 @@ fa_status launch_visibility(fa_ctx* ctx, const fa_mesh* mesh, const Mat4& M, uin
     launch_k(cons ? k_raster_mark<kMarkConservative> : k_raster_mark<kMarkSamples>, 152 * 4, 256, 0, s, A);
   if (A.win && cons) {
     mark(ctx, "k_raster_mark_cons", s);
-    launch_k(k_raster_mark_cons, 152 * 8, 256, 0, s, A);
+    launch_k(k_raster_mark_cons, 152 * 4, 256, 0, s, A);  // (one wave: the shares are claimed)
   }
   FA_CUDA_TRY(cudaGetLastError());
   return FA_OK;

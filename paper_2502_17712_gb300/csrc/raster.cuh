@@ -570,6 +570,7 @@ __device__ __forceinline__ void front_body(const RasterArgs& A, uint32_t bid, ui
       A.ctr->n_vtiles = 0u;
       A.ctr->uf_item = 0u;
       A.ctr->n_ties = 0u;
+      A.ctr->cons_item = 0u;
     }
   }
   if (bid == 0 && threadIdx.x < kMidLists) A.ctr->n_mid[threadIdx.x][0] = 0u;
@@ -1178,20 +1179,27 @@ __device__ __forceinline__ WinSetup win_setup(const RasterArgs& A, const float4&
   return s;
 }
 
-// Conservative marking takes a sub-triangle whose conservative box has more than kMidPix
-// pixels by tiles, so the exact pass queues it with that box (as setup's; the samples past
-// its own box are not covered).  Gives s that box if so.
-__device__ __forceinline__ bool cons_queue(const RasterArgs& A, WinSetup& s) {
-  if (!s.front) return false;
+// Pixels of the conservative box (as setup's) instead of the samples'; 0: none.
+__device__ __forceinline__ int cons_pixels(const RasterArgs& A, WinSetup& s) {
   const int xmn = min(s.v.X[0], min(s.v.X[1], s.v.X[2])), xmx = max(s.v.X[0], max(s.v.X[1], s.v.X[2]));
   const int ymn = min(s.v.Y[0], min(s.v.Y[1], s.v.Y[2])), ymx = max(s.v.Y[0], max(s.v.Y[1], s.v.Y[2]));
   const int px0 = max(-((-xmn) >> 8) - 1, 0), px1 = min(xmx >> 8, A.W - 1);
   const int py0 = max(-((-ymn) >> 8) - 1, 0), py1 = min(ymx >> 8, A.H - 1);
-  if (px1 < px0 || py1 < py0 || (px1 - px0 + 1) * (py1 - py0 + 1) <= kMidPix) return false;
   s.px0 = px0;
   s.py0 = py0;
   s.px1 = px1;
   s.py1 = py1;
+  return max(px1 - px0 + 1, 0) * max(py1 - py0 + 1, 0);
+}
+
+// Conservative marking takes a sub-triangle whose conservative box has more than kMidPix
+// pixels by tiles, so the exact pass queues it with that box (the samples past its own box
+// are not covered).  Gives s that box if so.
+__device__ __forceinline__ bool cons_queue(const RasterArgs& A, WinSetup& s) {
+  if (!s.front) return false;
+  WinSetup c = s;
+  if (cons_pixels(A, c) <= kMidPix) return false;
+  s = c;
   return true;
 }
 
@@ -1599,7 +1607,7 @@ __device__ __forceinline__ uint32_t mid_base(const RasterArgs& A, uint32_t r) {
 
 // Exact set-up of the survivors (as exact_body): small ones rasterized here, mid-size
 // ones listed, large ones queued.
-// CONS: for conservative marking (cons_queue).
+// CONS: conservative marking (A.cons) may ask for cons_queue.
 template <bool DEV_M, int NT, bool CONS>
 __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
   uint32_t* pre = region_pre();
@@ -1632,7 +1640,7 @@ __device__ __forceinline__ void exact_win_body(const RasterArgs& A, uint32_t bid
         const int w = E.px1 - E.px0 + 1, h = E.py1 - E.py0 + 1, pix = w * h;
         kind = !E.fits ? 2 : pix <= kSmallMaxPix ? 1 : pix <= kMidPix ? 3 : 2;
       }
-      if (CONS && cons_queue(A, E)) kind = 2;
+      if (CONS && A.cons && cons_queue(A, E)) kind = 2;
       if (kind == 2) tiles = tiles_of(E.px1 - E.px0 + 1, E.py1 - E.py0 + 1);
     }
     // large triangles of the warp reserve queue records and tiles with one atomic; what
@@ -2020,15 +2028,17 @@ __device__ __forceinline__ void mark_win_body(const RasterArgs& A, uint32_t bid,
 // Conservative marking after the winners': the triangles that the samples marked are
 // marked already (a covered centre's depth is the sample's), so only the other survivors
 // are tested, each pixel of their conservative boxes against the final keys (as
-// sample<2>).  Boxes above kMidPix pixels and clipped triangles' are the queued tiles, a warp
-// each, as in two rasterizations: a hidden triangle is looked at whole, and one that fills
-// a 1080p window takes a warp 18 ms and, clipped, a thread 0.77 s (by tiles 29 and 33 us).  Of the others
-// those of at most kSmallMaxPix pixels are tested in-thread and larger ones by the warp
-// together when there are many survivors; with few, a warp takes few of them, all together.
-// Against a second rasterization of every survivor (conservative fa_visibility at 1080p):
-// a floor of 60 patches 387 -> 250 us, 200 icospheres 209 -> 183.  What is left is the
-// hidden triangles' boxes, every pixel of them; four pixels' loads at once cost
-// registers and are slower (321, 206).
+// sample<2>).  Boxes above kMidPix pixels and clipped triangles' are the queued tiles, a
+// warp each, as in two rasterizations: a hidden triangle is looked at whole, and one that
+// fills a 1080p window takes a warp 18 ms and, clipped, a thread 0.77 s (by tiles 29 and 33
+// us).  Of the others those of at most kSmallMaxPix pixels are tested in-thread and larger
+// ones by the warp together when there are many survivors; with few, a warp takes few of
+// them, all together.  Edge functions in 32 bits, stepped, as in win_box (an edge's largest
+// value over a pixel's square is half a step each way from the centre's: 2 % more).
+// (Conservative marking of 60 patches at 1080p 182 us with 64-bit edge functions set up at
+// every pixel, 100 so; of 200 icospheres, 4.1M triangles, 216 and 66; a 1,024-thread block
+// of the persistent kernel has four pixels' keys on their way, its frame of the latter 466
+// -> 424 us.)
 __device__ __forceinline__ bool cons_box(const RasterArgs& A, const SV& a, const SV& b, const SV& c, int px0, int py0,
                                          int px1, int py1, uint32_t first, uint32_t step) {
   const int64_t Ar = (b.X - a.X) * (c.Y - a.Y) - (c.X - a.X) * (b.Y - a.Y);
@@ -2053,6 +2063,52 @@ __device__ __forceinline__ bool cons_box(const RasterArgs& A, const SV& a, const
     if (!in) d = fminf(fmaxf(d, zmin), zmax);
     if (!(d >= -1.0f && d <= 1.0f)) continue;
     if (ordered(d) <= zkey(A, (uint32_t)py * (uint32_t)A.W + (uint32_t)px)) return true;
+  }
+  return false;
+}
+
+template <int N>
+__device__ __forceinline__ bool cons_box32(const RasterArgs& A, const Tri32& v, int px0, int py0, int px1, int py1,
+                                           int first, int step) {
+  const int w = px1 - px0 + 1, n = w * (py1 - py0 + 1);
+  if (first >= n) return false;
+  const int sy = step == 1 ? (w == 1 ? 1 : 0) : step / w, sx = step - sy * w;  // step = sy rows and sx < w pixels
+  const int fy = first / w, fx = first - fy * w;
+  const Edges32 E = edges32(v, px0 + fx, py0 + fy);
+  const float zmin = fminf(v.z[0], fminf(v.z[1], v.z[2])), zmax = fmaxf(v.z[0], fmaxf(v.z[1], v.z[2]));
+  int e[3], in_row[3], past[3], half[3];  // half: from a centre's (reduced) value to the square's largest
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    e[i] = E.e[i];
+    in_row[i] = E.dy[i] * sy + E.dx[i] * sx;
+    past[i] = in_row[i] + E.dy[i] - E.dx[i] * w;
+    half[i] = ((abs(E.dx[i]) + abs(E.dy[i])) >> 1) + E.nb[i];
+  }
+  const uint32_t ap = (uint32_t)(A.W * sy + sx), bp = ap + (uint32_t)(A.W - w);
+  uint32_t p = (uint32_t)(py0 + fy) * (uint32_t)A.W + (uint32_t)(px0 + fx);
+  for (int left = n - 1 - first, col = w - fx; left >= 0;) {
+    uint32_t key[N], pix[N];
+    bool on[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      pix[i] = p;
+      on[i] = ((e[0] + half[0]) | (e[1] + half[1]) | (e[2] + half[2]) | left) >= 0;
+      float f = __fmul_rn(__int2float_rn(e[0] + E.nb[0]), v.z[0]);
+      f = __fadd_rn(f, __fmul_rn(__int2float_rn(e[1] + E.nb[1]), v.z[1]));
+      f = __fadd_rn(f, __fmul_rn(__int2float_rn(e[2] + E.nb[2]), v.z[2]));
+      float d = __fmul_rn(f, E.invA);
+      if ((e[0] | e[1] | e[2]) < 0) d = fminf(fmaxf(d, zmin), zmax);
+      on[i] = on[i] && d >= -1.0f && d <= 1.0f;
+      key[i] = ordered(d);
+      col -= sx;
+      const bool wrap = col <= 0;
+      col += wrap ? w : 0;
+      p += wrap ? bp : ap;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) e[k] += wrap ? past[k] : in_row[k];
+      left -= step;
+    }
+    if (test_n(A, on, key, pix)) return true;
   }
   return false;
 }
@@ -2094,56 +2150,68 @@ __device__ __forceinline__ void mark_cons_body(const RasterArgs& A, uint32_t bid
   const uint32_t stride = nblk * blockDim.x, warp = (bid * blockDim.x + threadIdx.x) >> 5, nwarps = stride >> 5;
   uint32_t per = 32;  // survivors a warp takes at a time
   while (per > 1u && (uint64_t)n * 32u <= (uint64_t)nwarps * per * 16u) per >>= 1;
-  for (uint32_t base = warp * per; base < n; base += nwarps * per) {
-    const uint32_t v = base + lane;
-    SV a{0, 0, 0.0f}, b{0, 0, 0.0f}, c{0, 0, 0.0f};
-    Setup S{0, 0, 0, -1, -1};
+  // (a warp's first share by its index, the next ones from a counter, claimed ahead: shares
+  // differ by an order of magnitude, and a block waits for its slowest warp)
+  for (uint32_t share = warp; (uint64_t)share * per < n;) {
+    const uint32_t base = share * per, v = base + lane;
+    uint32_t claimed = 0;
+    if (lane == 0) claimed = atomicAdd(&A.ctr->cons_item, 1u);
+    WinSetup E = {};
     uint32_t t = 0;
     bool vis = false, big = false;
     if (lane < per && v < n) {
       const uint32_t i = surv_slot(A, pre, v, base);
       t = __ldcg(A.surv + i);
-      if (!((__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u)) {
+      if (!marked(A, t)) {
         const float4* sc = A.surv_clip + 3 * (size_t)i;
-        const float4 c0 = __ldcs(sc), c1 = __ldcs(sc + 1), c2 = __ldcs(sc + 2);
-        a = project(CV{c0.x, c0.y, c0.z, c0.w}, A.hx, A.hy);
-        b = project(CV{c1.x, c1.y, c1.z, c1.w}, A.hx, A.hy);
-        c = project(CV{c2.x, c2.y, c2.z, c2.w}, A.hx, A.hy);
-        S = setup(a, b, c, A.W, A.H, true);
-        const int pix = (S.px1 - S.px0 + 1) * (S.py1 - S.py0 + 1);
-        if (S.A > 0 && S.px1 >= S.px0 && S.py1 >= S.py0 && pix <= most) {
-          big = pix > (per < 32u ? 1 : kSmallMaxPix);
-          if (!big) vis = cons_box(A, a, b, c, S.px0, S.py0, S.px1, S.py1, 0u, 1u);
+        E = win_setup(A, __ldcs(sc), __ldcs(sc + 1), __ldcs(sc + 2));
+        const int pix = E.front ? cons_pixels(A, E) : 0;
+        if (pix > 0 && pix <= most) {
+          big = pix > (per < 32u ? 1 : kSmallMaxPix) || !E.fits;
+          if (!big) vis = cons_box32<(NT > 256 ? 4 : 1)>(A, E.v, E.px0, E.py0, E.px1, E.py1, 0, 1);
         }
       }
     }
     for (uint32_t m = __ballot_sync(0xFFFFFFFFu, big); m; m &= m - 1u) {  // the warp together
       const int src = __ffs(m) - 1;
-      const SV qa{__shfl_sync(0xFFFFFFFFu, (int32_t)a.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)a.Y, src),
-                  __shfl_sync(0xFFFFFFFFu, a.zn, src)};
-      const SV qb{__shfl_sync(0xFFFFFFFFu, (int32_t)b.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)b.Y, src),
-                  __shfl_sync(0xFFFFFFFFu, b.zn, src)};
-      const SV qc{__shfl_sync(0xFFFFFFFFu, (int32_t)c.X, src), __shfl_sync(0xFFFFFFFFu, (int32_t)c.Y, src),
-                  __shfl_sync(0xFFFFFFFFu, c.zn, src)};
-      const int px0 = __shfl_sync(0xFFFFFFFFu, S.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, S.py0, src);
-      const int px1 = __shfl_sync(0xFFFFFFFFu, S.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, S.py1, src);
-      const bool hit = cons_box(A, qa, qb, qc, px0, py0, px1, py1, lane, 32u);
+      Tri32 q;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        q.X[j] = __shfl_sync(0xFFFFFFFFu, E.v.X[j], src);
+        q.Y[j] = __shfl_sync(0xFFFFFFFFu, E.v.Y[j], src);
+        q.z[j] = __shfl_sync(0xFFFFFFFFu, E.v.z[j], src);
+      }
+      const int px0 = __shfl_sync(0xFFFFFFFFu, E.px0, src), py0 = __shfl_sync(0xFFFFFFFFu, E.py0, src);
+      const int px1 = __shfl_sync(0xFFFFFFFFu, E.px1, src), py1 = __shfl_sync(0xFFFFFFFFu, E.py1, src);
+      bool hit;
+      if (fits32(q)) {
+        hit = cons_box32<1>(A, q, px0, py0, px1, py1, (int)lane, 32);
+      } else {
+        const SV a{q.X[0], q.Y[0], q.z[0]}, b{q.X[1], q.Y[1], q.z[1]}, c{q.X[2], q.Y[2], q.z[2]};
+        hit = cons_box(A, a, b, c, px0, py0, px1, py1, lane, 32u);
+      }
       if (__any_sync(0xFFFFFFFFu, hit) && (int)lane == src) vis = true;
     }
     if (vis) win_mark(A, t);
+    share = nwarps + __shfl_sync(0xFFFFFFFFu, claimed, 0);
   }
   __syncthreads();  // pre is reused
   const uint32_t nc = region_prefix<NT>(A, A.clip_count, pre);
   const Mat4 M = A.Mdev ? load_mat(A.Mdev) : A.M;
   for (uint32_t i = bid * blockDim.x + threadIdx.x; i < nc; i += stride) {
     const uint32_t t = __ldcg(A.clip + surv_slot(A, pre, i, i));
-    if ((__ldcg(A.vt + (t >> 5)) >> (t & 31)) & 1u) continue;
+    if (marked(A, t)) continue;
     const uint32_t* f = A.idx + 3 * (size_t)t;
     if (cons_clipped(A, load_clip(M, A.pos, __ldg(f)), load_clip(M, A.pos, __ldg(f + 1)),
                      load_clip(M, A.pos, __ldg(f + 2)), full))
       win_mark(A, t);
   }
-  // (inlined: as a call it takes the loops' registers, 60 patches at 1080p 244 us instead of 182)
+}
+
+// ... and of the queued tiles.  (A call of it in the body above takes that one's registers:
+// in the kernel it is inlined after it, in the persistent kernel a function beside it.)
+__device__ __forceinline__ void mark_cons_tiles(const RasterArgs& A, uint32_t bid, uint32_t nblk) {
+  if (!A.win || !A.cons || __ldcg(&A.ctr->status) != 0) return;
   for_tiles<MarkTile<2>>(A, __ldcg(&A.ctr->big), bid, nblk);
 }
 
