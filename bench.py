@@ -180,17 +180,17 @@ def algorithmic_bytes(kernel, T, V, W, H, T_vis, C, work=None):
     n_vtiles = w.get("visible_tiles", (T + 1023) // 1024)
     n_blocks = (T + 1023) // 1024
     table = {
-        # read indices + positions once; clear the depth buffer (counted as keys alone:
-        # the triangle kept beside each key is not compulsory), VT and tri_chart
+        # read indices + positions once; clear the depth buffer (one word a pixel here and
+        # below: of key and triangle only one is compulsory), VT and tri_chart
         "k_raster_front": 12 * T + 12 * V + 4 * W * H + vt + 4 * T,
         # read each survivor (id + clip coordinates), the depth buffer written once
-        "k_raster_exact": (4 + 48) * n_surv + 8 * W * H,
+        "k_raster_exact": (4 + 48) * n_surv + 4 * W * H,
         # read the queue records and tile owners (the mid-size records are not counted)
         "k_raster_depth_big": 64 * n_big + 4 * n_tiles,
         # read the depth buffer once, write the largest key of each 16x16 tile
         "k_raster_zmax": 4 * W * H + 4 * ((W + 15) // 16) * ((H + 15) // 16),
         # the depth buffer read once, VT written once
-        "k_raster_mark": 8 * W * H + vt,
+        "k_raster_mark": 4 * W * H + vt,
         # per chart: box + full flag read, footprint + rotation written, rank written
         "k_order_tile": C * (16 + 4 + 12 + 4),
         # per chart: rank + footprint read, order, sorted footprint and position written

@@ -360,8 +360,9 @@ fa_status fa_set_wait_limits(fa_ctx* ctx, uint32_t loop_cap, uint64_t wait_ns);
 
 /* Raster schedule of this context's later frames (changes timing only, never
  * results).  By default a frame is rasterized once (the depth pass keeps each pixel's
- * triangle; conservative marking then tests what the samples left unmarked); with
- * FA_RASTER_HIZ it is rasterized a second time to mark, and mid_max_pix applies then.
+ * triangle; conservative marking then tests what the samples left unmarked), and
+ * mid_max_pix changes nothing; with FA_RASTER_HIZ it is rasterized a second time to
+ * mark, and mid_max_pix applies then.
  *  mid_max_pix: a sub-triangle whose pixel box has at most 16 pixels is rasterized
  *    by one thread; larger ones are split into 16x16 tiles, one warp per tile.
  *    With mid_max_pix > 16, boxes of up to mid_max_pix pixels are also rasterized
@@ -375,8 +376,8 @@ fa_status fa_set_wait_limits(fa_ctx* ctx, uint32_t loop_cap, uint64_t wait_ns);
  *    skips a sub-triangle (or a tile of one) whose smallest possible sample depth, less
  *    a bound on the depth's rounding error, is above the largest depth of every tile it
  *    touches.  Off by default: one rasterization is faster on every scene measured (64
- *    views of overlapping floors one after the other: 17.5 ms, 27.2 with the option and
- *    mid_max_pix 64).
+ *    views of overlapping floors one after the other: 17.4 ms, 26.9 with the option and
+ *    mid_max_pix 64) but small ones of coincident geometry, where the two are close.
  * Both ways the same samples get the same depth keys and the same triangles are
  * marked.  Errors: FA_E_INVALID_ARG (NULL ctx, mid_max_pix outside [16, 256],
  * unknown flags). */
@@ -421,9 +422,12 @@ typedef struct fa_frame_stats {
   uint32_t survivors;     /* triangles that passed the raster front end */
   uint32_t clipped;       /* of those, triangles that needed clipping */
   uint32_t clip_records;  /* small sub-triangle records of the clipping path (FA_RASTER_HIZ; else 0) */
-  uint32_t big_entries;   /* large sub-triangles queued for tile rasterization */
+  uint32_t big_entries;   /* large sub-triangles queued for tile rasterization: boxes of more than 256
+                             pixels (conservative ones with FA_VIS_CONSERVATIVE) or 96 pixels a side,
+                             clipped ones of more than 16; all of more than 16 with FA_RASTER_HIZ */
   uint64_t big_tiles;     /* their 16x16 tiles */
-  uint32_t visible;       /* entries of the visible-triangle list */
+  uint32_t visible;       /* entries of the last chart pass's visible-triangle list (fa_parameterize and
+                             fa_uv alone walk the caller's chart ids and leave it) */
   uint32_t charts;        /* charts of the last chart pass */
   uint32_t visible_tiles; /* tiles of 1024 consecutive triangles holding a visible one */
 } fa_frame_stats;
